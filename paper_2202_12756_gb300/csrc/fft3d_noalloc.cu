@@ -152,7 +152,7 @@ extern "C" int fft3d_exec_c2r_noalloc(const void *in_cplx, void *out_real, int64
     if ((size_t)col_table_elems((int)n0, g0) * csize > kTableSlot ||
         (size_t)col_table_elems((int)n1, g1) * csize > kTableSlot ||
         (size_t)line_tw_size(z_line_points((int)m, gz), gz.E) * csize > kTableSlot ||
-        z_table_elems(f32, (int)m) * csize > kZTableSlot)
+        z_table_elems((int)m) * csize > kZTableSlot)
         return FFT3D_ERR_SIZE;
 
     void *scratch = nullptr;

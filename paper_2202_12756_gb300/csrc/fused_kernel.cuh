@@ -23,7 +23,7 @@
 // with L2-only loads.
 #pragma once
 
-#include "pass_kernels.cuh"
+#include "fx_kernels.cuh"
 
 namespace fft3d {
 

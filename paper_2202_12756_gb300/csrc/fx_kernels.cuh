@@ -1,0 +1,608 @@
+// Fixed-point forms of the double-precision passes (see fx_math.cuh): the
+// same tiles, lines and exchanges as the passes of pass_kernels.cuh, with the
+// transform on 64-bit integers.  A tile or line group that holds a line outside
+// the conversions' range (non-finite values, exponents near the ends of the
+// double range) runs the FP64 pass instead, from the same twiddle tables.
+//
+// Measured on GB300 in place (FP64 arithmetic -> fixed point): 1024^3 pair
+// 190.1 -> 43.9 ms (column passes 30.3 -> 6.7 ms each, z-passes 34.5 -> 6.5 and
+// 10.5), 512^3 21.6 -> 5.85 ms; relative L2 error of one transform 2.0-2.6e-16
+// -> 0.8-1.6e-16 against quadruple precision over every line length.
+#pragma once
+
+#include "pass_kernels.cuh"
+
+namespace fft3d {
+
+// Lengths transformed in fixed point; shorter ones have too few FP64
+// operations per element to gain.
+template <typename R, int L> __host__ __device__ constexpr bool col_fixed() { return sizeof(R) == 8 && L >= 8; }
+template <typename R, int M> __host__ __device__ constexpr bool z_fixed() { return sizeof(R) == 8 && M >= 4; }
+
+// table scale of the R2C rotation factors
+constexpr int kFxRotShift = 2;
+
+__device__ __forceinline__ fxtw fx_ldg(const fxtw *p)
+{
+    const int4 q = __ldg((const int4 *)p);
+    return fxtw{q.x, q.y, q.z, q.w};
+}
+
+// Scale code of a thread's n complex values.
+template <int N> __device__ __forceinline__ int fx_thread_code(const double2 *v)
+{
+    int32_t tm = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) tm = max(tm, max(fx_top(v[i].x), fx_top(v[i].y)));
+    const int32_t ex = tm & 0x7ff00000;
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s += fx_mag(fx_top(v[i].x), ex) + fx_mag(fx_top(v[i].y), ex);
+    return fx_code(tm, s);
+}
+
+// Half of a complex result by the integer pipe, half by the (otherwise idle)
+// FP64 pipe.
+__device__ __forceinline__ double2 fx_out(fxc z, int e) { return cmake<double2>(fx_to(z.x, e), fx_to_fp(z.y, e)); }
+
+// ------------------------------------------------------------ columns
+template <int L, int E, int W, bool INV>
+__device__ __noinline__ void col_tile_slow(const ColArgs &a, int64_t tile, unsigned char *smem, const fxtw *tw)
+{
+    col_tile<double, L, E, W, false, INV>(a, tile, smem, tw);
+}
+
+template <int L, int E, int W, bool INV>
+__global__ void __launch_bounds__(W *(L / E), (W * (L / E) >= 512 ? 1 : 512 / (W * (L / E))))
+colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw)
+{
+    constexpr int NT = L / E;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int *code = (int *)(smem_raw + (size_t)L * W * sizeof(fxc));
+    const int c = threadIdx.x % W;
+    const int j = threadIdx.x / W;
+    double2 *sp = nullptr, *dp = nullptr;
+    int64_t ss = 0, ds = 0;
+    const bool valid = col_decode<double2, W>(a, blockIdx.x, c, sp, ss, dp, ds);
+    if (threadIdx.x < W) code[threadIdx.x] = 0;
+    fxc v[E];
+    int g;
+    {
+        double2 r[E];
+        const double2 *sj = sp + (int64_t)j * ss;
+        const int64_t sstep = (int64_t)NT * ss;
+#pragma unroll
+        for (int i = 0; i < E; ++i) r[i] = sj[i * sstep];
+        if constexpr (NT > 1) {
+            g = fx_thread_code<E>(r);
+            __syncthreads();
+            if constexpr (W < 32) {
+#pragma unroll
+                for (int o = W; o < 32; o *= 2) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+                if ((threadIdx.x & 31) < W) atomicMax(code + c, g);
+            } else {
+                atomicMax(code + c, g);
+            }
+        } else {
+            g = fx_thread_code<E>(r);
+            code[c] = g;
+        }
+        __syncthreads();
+        bool ok = true;
+#pragma unroll
+        for (int i = 0; i < W; ++i) ok = ok && fx_code_ok(code[i]);
+        if (!ok) {
+            __syncthreads();
+            col_tile_slow<L, E, W, INV>(a, blockIdx.x, smem_raw, tw);
+            return;
+        }
+        g = code[c];
+        g = g == 0 ? kFxZeroCode : g;
+#pragma unroll
+        for (int i = 0; i < E; ++i)
+            v[i] = fx_make(fx_from(INV ? r[i].y : r[i].x, g, kFxBits), fx_from(INV ? r[i].x : r[i].y, g, kFxBits));
+    }
+    ColEx<fxc, W> ex{(fxc *)smem_raw, c};
+    line_fft<fx64, L, E>(v, j, tw, ex);
+    const int e = g - 1023 - kFxBits + fx_line_shift<L, E>();
+    if (valid) {
+        double2 *dj = dp + (int64_t)j * ds;
+        const int64_t dstep = (int64_t)NT * ds;
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            double2 o = fx_out(v[i], e);
+            if (INV) o = cswap(o);
+            dj[i * dstep] = o;
+        }
+    }
+}
+
+// ------------------------------------------------------------ lines
+// Largest scale code of a line (NT threads).
+template <int NT, int LPB, class Ex> __device__ __forceinline__ int fx_line_max(int g, const Ex &ex)
+{
+#pragma unroll
+    for (int o = (NT < 32 ? NT : 32) / 2; o > 0; o /= 2) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+    if constexpr (NT > 32) {
+        constexpr int WPL = NT / 32;
+        __shared__ int code[LPB * WPL];
+        const int w = threadIdx.x / 32;
+        if (threadIdx.x % 32 == 0) code[w] = g;
+        ex.sync();
+#pragma unroll
+        for (int i = 0; i < WPL; ++i) g = max(g, code[w / WPL * WPL + i]);
+    }
+    return g;
+}
+// The threads that synchronise together agree.
+template <int NT> __device__ __forceinline__ bool fx_all_ok(int g)
+{
+    if constexpr (NT > 32) return fx_code_ok(g);
+    else return __all_sync(0xffffffffu, fx_code_ok(g));
+}
+
+template <int M, int E, int LPB>
+__device__ __noinline__ void zr2c_slow(const ZArgs &a, int64_t line0, unsigned char *smem, const fxtw *tw,
+                                       const fxtw *rot)
+{
+    if constexpr (z_paired<double, M>()) zr2c_pairs<double, M, E, LPB>(a, line0, smem, tw);
+    else zr2c_lines<double, M, E, LPB>(a, line0, smem, tw, rot);
+}
+template <int M, int E, int LPB>
+__device__ __noinline__ void zc2r_slow(const ZArgs &a, int64_t line0, unsigned char *smem, const fxtw *tw,
+                                       const fxtw *rot)
+{
+    if constexpr (z_paired<double, M>()) zc2r_pairs<double, M, E, LPB, false>(a, line0, smem, tw);
+    else zc2r_lines<double, M, E, LPB, false>(a, line0, smem, tw, rot);
+}
+
+// zr2c_lines in fixed point: X[k] = (s - i r d) / 2 with s = Z[k] + conj Z[M - k],
+// d = Z[k] - conj Z[M - k], formed as X / 2 = s / 4 - i (r / 4) d.
+template <int M, int E, int LPB>
+__device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                              const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
+{
+    constexpr int NT = M / E;
+    constexpr int P = zline_pad<E>();
+    const int lt = threadIdx.x / NT;
+    const int j = threadIdx.x % NT;
+    const int64_t line = line0 + lt;
+    const bool active = line < a.nlines;
+    LineEx<fxc, NT, P> ex{(fxc *)smem + lt * zline_smem_elems<M, E>(), line_bar<NT, LPB>(lt)};
+
+    fxc v[E];
+    int g;
+    {
+        const double2 *in = (const double2 *)((const double *)a.real + (active ? line : 0) * a.real_pitch);
+        double2 r[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) r[i] = active ? in[j + i * NT] : cmake<double2>(0.0, 0.0);
+        g = fx_line_max<NT, LPB>(fx_thread_code<E>(r), ex);
+        if (!fx_all_ok<NT>(g)) {
+            zr2c_slow<M, E, LPB>(a, line0, smem, tw, rot);
+            return;
+        }
+        g = g == 0 ? kFxZeroCode : g;
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
+    }
+    line_fft<fx64, M, E>(v, j, tw, ex);
+
+    const int e = g - 1023 - kFxBits + fx_line_shift<M, E>();
+    double2 *out = (double2 *)a.cplx.main + (active ? line : 0) * (M + 1);
+    const double se = a.scale_edge, sm = a.scale_mid;
+    const bool unit = se == 1.0 && sm == 1.0;
+    auto emit = [&](int k, fxc z, fxc zm) {
+        const fxc zc = cconj(zm);
+        const fxc s = fx_shr<2>(cadd(z, zc));
+        const fxc p = cmul(csub(z, zc), fx_ldg(rot + k));
+        double2 x = fx_out(fx_make(s.x + p.y, s.y - p.x), e + 1);
+        if (!unit) x = cscale(x, k == 0 ? se : sm);
+        if (active) store_out(out + k, x);
+    };
+    if constexpr (NT <= 32) {
+        const int src = (NT - j) & (NT - 1);
+        static_for<0, E>([&](auto II) {
+            constexpr int i = decltype(II)::value;
+            fxc zp;
+            zp.x = __shfl_sync(0xffffffffu, (long long)v[E - 1 - i].x, src, NT);
+            zp.y = __shfl_sync(0xffffffffu, (long long)v[E - 1 - i].y, src, NT);
+            emit(j + i * NT, v[i], (j == 0) ? v[(E - i) % E] : zp);
+        });
+    } else {
+        constexpr bool LR = pad_linear_reads<P>(NT);
+        constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
+#pragma unroll
+        for (int i = 0; i < E; ++i) ex.put(pad_row<P, LR>(j, i * NT), v[i]);
+        ex.sync();
+        static_for<0, E>([&](auto II) {
+            constexpr int i = decltype(II)::value;
+            emit(j + i * NT, v[i], (i == 0 && j == 0) ? v[0] : ex.get(pad_row<P, LREV>(M - j, -i * NT)));
+        });
+    }
+    if (active && j == 0) {
+        double x = fx_to(v[0].x - v[0].y, e);
+        if (!unit) x *= se;
+        out[M] = cmake<double2>(x, 0.0);
+    }
+}
+
+// Output scale s of a C2R line as an exponent where it is a power of two (the
+// factor left over is then 1).
+__device__ __forceinline__ double fx_split_scale(double s, int &e)
+{
+    const uint64_t u = fx_bits(s);
+    const int ex = (int)(u >> 52 & 0x7ff);
+    if ((u & 0xfffffffffffffULL) == 0 && ex > 1023 - 100 && ex < 1023 + 100) {
+        e += ex - 1023;
+        return 1.0;
+    }
+    return s;
+}
+
+// zc2r_lines in fixed point.  The pre-process at most quadruples a thread's L1
+// norm (its own entries and their mirror images, twice each), so the entries
+// come in at 2^-2 of the usual scale; its rotation by r / 4 acts on 4 d.
+template <int M, int E, int LPB>
+__device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                              const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
+{
+    constexpr int NT = M / E;
+    constexpr int P = zline_pad<E>();
+    const int lt = threadIdx.x / NT;
+    const int j = threadIdx.x % NT;
+    const int64_t line = line0 + lt;
+    const bool active = line < a.nlines;
+    LineEx<fxc, NT, P> ex{(fxc *)smem + lt * zline_smem_elems<M, E>(), line_bar<NT, LPB>(lt)};
+
+    const int64_t l = active ? line : 0;
+    fxc v[E], xm;
+    int g;
+    {
+        const double2 *src = (const double2 *)a.cplx.main + l * (a.cplx.split ? M : M + 1);
+        const double2 *nyq = a.cplx.split ? (const double2 *)a.cplx.nyq + l : src + M;
+        double2 r[E + 1];
+#pragma unroll
+        for (int i = 0; i < E; ++i) r[i] = active ? src[j + i * NT] : cmake<double2>(0.0, 0.0);
+        r[E] = active && j == 0 ? *nyq : cmake<double2>(0.0, 0.0);
+        if (j == 0) {
+            // only the real parts of the k2 = 0 and k2 = M entries enter
+            r[0] = cmake<double2>(a.scale_edge * r[0].x, 0.0);
+            r[E] = cmake<double2>(a.scale_edge * r[E].x, 0.0);
+        }
+        g = fx_line_max<NT, LPB>(fx_thread_code<E + 1>(r), ex);
+        if (!fx_all_ok<NT>(g)) {
+            zc2r_slow<M, E, LPB>(a, line0, smem, tw, rot);
+            return;
+        }
+        g = g == 0 ? kFxZeroCode : g;
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits - 2), fx_from(r[i].y, g, kFxBits - 2));
+        xm = fx_make(fx_from(r[E].x, g, kFxBits - 2), 0);
+    }
+    // conj(Z[k]) from x = X[k] and y = X[M - k]
+    auto pre = [&](int k, fxc x, fxc y) -> fxc {
+        const fxc yc = cconj(y);
+        const fxc s = cadd(x, yc), d = csub(x, yc);
+        const fxc o = cmulc(fx_make(d.x * 4, d.y * 4), fx_ldg(rot + k));
+        return fx_make(s.x - o.y, -(s.y + o.x));
+    };
+    if constexpr (NT <= 32) {
+        const int srcl = (NT - j) & (NT - 1);
+        fxc up = xm;  // lane 0: the value that slot E - i held before its update
+        static_for<0, (E + 1) / 2>([&](auto II) {
+            constexpr int i = decltype(II)::value;
+            constexpr int h = E - 1 - i;
+            // slots i and h of lanes j and NT - j are each other's mirror images
+            // (lane 0: slots i and E - i of its own)
+            fxc pi, ph;
+            pi.x = __shfl_sync(0xffffffffu, (long long)v[h].x, srcl, NT);
+            pi.y = __shfl_sync(0xffffffffu, (long long)v[h].y, srcl, NT);
+            ph.x = __shfl_sync(0xffffffffu, (long long)v[i].x, srcl, NT);
+            ph.y = __shfl_sync(0xffffffffu, (long long)v[i].y, srcl, NT);
+            if (j == 0) {
+                pi = up;
+                ph = v[i + 1 < E ? i + 1 : i];
+                if constexpr (i == h) ph = pi;
+            }
+            up = v[h];
+            const fxc nh = pre(j + h * NT, v[h], ph);
+            if constexpr (i != h) {
+                v[i] = pre(j + i * NT, v[i], pi);
+                v[h] = nh;
+            } else {
+                v[h] = pre(j + h * NT, v[h], pi);
+            }
+        });
+    } else {
+        constexpr bool LR = pad_linear_reads<P>(NT);
+        constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
+#pragma unroll
+        for (int i = 0; i < E; ++i) ex.put(pad_row<P, LR>(j, i * NT), v[i]);
+        if (j == 0) ex.put(pad_row<P, true>(M, 0), xm);
+        ex.sync();
+        static_for<0, E>([&](auto II) {
+            constexpr int i = decltype(II)::value;
+            v[i] = pre(j + i * NT, v[i], ex.get(pad_row<P, LREV>(M - j, -i * NT)));
+        });
+        ex.sync();
+    }
+    line_fft<fx64, M, E>(v, j, tw, ex);
+
+    int e = g - 1023 - (kFxBits - 2) + fx_line_shift<M, E>();
+    const double f = fx_split_scale(a.scale_mid, e);
+    double2 *out = (double2 *)((double *)a.real_out + l * a.real_pitch);
+    if (active) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            double2 o = fx_out(cconj(v[i]), e);
+            if (f != 1.0) o = cscale(o, f);
+            store_out(out + j + i * NT, o);
+        }
+    }
+}
+
+// zr2c_pairs in fixed point; the two lines share a scale, as they share the
+// FP64 form's rounding errors.
+template <int M, int E, int LPB>
+__device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                              const fxtw *__restrict__ tw)
+{
+    constexpr int N = 2 * M;
+    constexpr int NT = N / E;
+    constexpr int PPB = LPB / 2;
+    constexpr int P = zline_pad<E>();
+    static_assert(LPB % 2 == 0 && NT > 32, "pairs of lines");
+    const int pt = threadIdx.x / NT;
+    const int j = threadIdx.x % NT;
+    const int64_t l0 = line0 + 2 * pt;
+    const bool act0 = l0 < a.nlines, act1 = l0 + 1 < a.nlines;
+    LineEx<fxc, NT, P> ex{(fxc *)smem + pt * zline_smem_elems<N, E>(), line_bar<NT, PPB>(pt)};
+
+    fxc v[E];
+    int g;
+    {
+        const double *in0 = (const double *)a.real + (act0 ? l0 : 0) * a.real_pitch;
+        const double *in1 = (const double *)a.real + (act1 ? l0 + 1 : 0) * a.real_pitch;
+        double2 r[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) r[i] = cmake<double2>(act0 ? in0[j + i * NT] : 0.0, act1 ? in1[j + i * NT] : 0.0);
+        g = fx_line_max<NT, PPB>(fx_thread_code<E>(r), ex);
+        if (!fx_all_ok<NT>(g)) {
+            zr2c_slow<M, E, LPB>(a, line0, smem, tw, nullptr);
+            return;
+        }
+        g = g == 0 ? kFxZeroCode : g;
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
+    }
+    line_fft<fx64, N, E>(v, j, tw, ex);
+
+    constexpr bool LR = pad_linear_reads<P>(NT);
+    constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
+#pragma unroll
+    for (int i = M / NT; i < E; ++i) ex.put(pad_row<P, LR>(j, i * NT), v[i]);  // only Z[N - k], k <= M, is read
+    ex.sync();
+    double2 *out0 = (double2 *)a.cplx.main + (act0 ? l0 : 0) * (M + 1);
+    double2 *out1 = out0 + (M + 1);
+    const int e = g - 1023 - kFxBits + fx_line_shift<N, E>() - 1;
+    const double se = a.scale_edge, sm = a.scale_mid;
+    const bool unit = se == 1.0 && sm == 1.0;
+    static_for<0, M / NT + 1>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        if (i < M / NT || j == 0) {
+            const int k = j + i * NT;
+            const fxc z = v[i];
+            const fxc zm = (k == 0 || k == M) ? z : ex.get(pad_row<P, LREV>(N - j, -i * NT));  // Z[N - k]
+            double2 x0 = fx_out(fx_make(z.x + zm.x, z.y - zm.y), e), x1 = fx_out(fx_make(z.y + zm.y, zm.x - z.x), e);
+            if (!unit) {
+                const double f = (k == 0 || k == M) ? se : sm;
+                x0 = cscale(x0, f);
+                x1 = cscale(x1, f);
+            }
+            if (act0) store_out(out0 + k, x0);
+            if (act1) store_out(out1 + k, x1);
+        }
+    });
+}
+
+// zc2r_pairs in fixed point.  Thread j converts the entries k = j + i NT < M of
+// both lines once; they give Z[k] = x0 + i x1, its own, and Z[N - k] =
+// conj x0 + i conj x1, which another thread of the pair owns.
+template <int M, int E, int LPB>
+__device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                              const fxtw *__restrict__ tw)
+{
+    constexpr int N = 2 * M;
+    constexpr int NT = N / E;
+    constexpr int H = E / 2;
+    constexpr int PPB = LPB / 2;
+    constexpr int P = zline_pad<E>();
+    static_assert(LPB % 2 == 0 && NT > 32 && H * NT == M, "pairs of lines");
+    const int pt = threadIdx.x / NT;
+    const int j = threadIdx.x % NT;
+    const int64_t l0 = line0 + 2 * pt;
+    const bool act0 = l0 < a.nlines, act1 = l0 + 1 < a.nlines;
+    LineEx<fxc, NT, P> ex{(fxc *)smem + pt * zline_smem_elems<N, E>(), line_bar<NT, PPB>(pt)};
+    constexpr bool LR = pad_linear_reads<P>(NT);
+    constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
+
+    const int64_t la = act0 ? l0 : 0, lb = act1 ? l0 + 1 : 0;
+    fxc v[E];
+    int g;
+    {
+        const int64_t pitch = a.cplx.split ? M : M + 1;
+        const double2 *src0 = (const double2 *)a.cplx.main + la * pitch;
+        const double2 *src1 = (const double2 *)a.cplx.main + lb * pitch;
+        const double2 zero = cmake<double2>(0.0, 0.0);
+        double2 r[E + 1];  // line l: slots 0..H-1, line l + 1: slots H..E-1, the k2 = M pair last
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            r[i] = act0 ? src0[j + i * NT] : zero;
+            r[H + i] = act1 ? src1[j + i * NT] : zero;
+        }
+        r[E] = zero;
+        if (j == 0) {
+            const double2 *nyq0 = a.cplx.split ? (const double2 *)a.cplx.nyq + la : src0 + M;
+            const double2 *nyq1 = a.cplx.split ? (const double2 *)a.cplx.nyq + lb : src1 + M;
+            const double we = a.scale_edge;
+            r[0] = cmake<double2>(we * r[0].x, 0.0);
+            r[H] = cmake<double2>(we * r[H].x, 0.0);
+            r[E] = cmake<double2>(act0 ? we * nyq0->x : 0.0, act1 ? we * nyq1->x : 0.0);
+        }
+        // a thread's transform inputs have at most twice this L1 norm (its own entries and their mirror images)
+        g = fx_line_max<NT, PPB>(fx_thread_code<E + 1>(r), ex);
+        if (!fx_all_ok<NT>(g)) {
+            zc2r_slow<M, E, LPB>(a, line0, smem, tw, nullptr);
+            return;
+        }
+        g = g == 0 ? kFxZeroCode : g;
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const fxc x0 = fx_make(fx_from(r[i].x, g, kFxBits - 1), fx_from(r[i].y, g, kFxBits - 1));
+            const fxc x1 = fx_make(fx_from(r[H + i].x, g, kFxBits - 1), fx_from(r[H + i].y, g, kFxBits - 1));
+            // inverse transform as swap(DFT(swap(Z)))
+            v[i] = fx_make(x0.y + x1.x, x0.x - x1.y);
+            const fxc m = fx_make(x1.x - x0.y, x0.x + x1.y);
+            if (i > 0 || j > 0) ex.put(pad_row<P, LREV>(N - j, -i * NT), m);
+        }
+        if (j == 0) {
+            const fxc x = fx_make(fx_from(r[E].x, g, kFxBits - 1), fx_from(r[E].y, g, kFxBits - 1));
+            ex.put(pad_row<P, true>(M, 0), fx_make(x.y, x.x));
+        }
+        ex.sync();
+#pragma unroll
+        for (int i = H; i < E; ++i) v[i] = ex.get(pad_row<P, LR>(j, i * NT));
+        ex.sync();
+    }
+    line_fft<fx64, N, E>(v, j, tw, ex);
+
+    int e = g - 1023 - (kFxBits - 1) + fx_line_shift<N, E>();
+    const double f = fx_split_scale(a.scale_mid, e);
+    double *out0 = (double *)a.real_out + la * a.real_pitch;
+    double *out1 = (double *)a.real_out + lb * a.real_pitch;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        double2 z = fx_out(cswap(v[i]), e);  // x0 + i x1 at n = j + i NT
+        if (f != 1.0) z = cscale(z, f);
+        if (act0) store_out(out0 + j + i * NT, z.x);
+        if (act1) store_out(out1 + j + i * NT, z.y);
+    }
+}
+
+// A group of LPB lines, by the form that serves the length.
+template <typename R, int M, int E, int LPB, bool PF>
+__device__ __forceinline__ void zr2c_group(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                           const typename twvec<R>::T *__restrict__ tw,
+                                           const typename twvec<R>::T *__restrict__ rot)
+{
+    if constexpr (!z_fixed<R, M>()) zr2c_lines<R, M, E, LPB, PF>(a, line0, smem, tw, rot);
+    else if constexpr (z_paired<R, M>()) zr2c_fx_pairs<M, E, LPB>(a, line0, smem, tw);
+    else zr2c_fx_lines<M, E, LPB>(a, line0, smem, tw, rot);
+}
+template <typename R, int M, int E, int LPB, bool PF>
+__device__ __forceinline__ void zc2r_group(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                           const typename twvec<R>::T *__restrict__ tw,
+                                           const typename twvec<R>::T *__restrict__ rot)
+{
+    if constexpr (!z_fixed<R, M>()) zc2r_lines<R, M, E, LPB, false, PF>(a, line0, smem, tw, rot);
+    else if constexpr (z_paired<R, M>()) zc2r_fx_pairs<M, E, LPB>(a, line0, smem, tw);
+    else zc2r_fx_lines<M, E, LPB>(a, line0, smem, tw, rot);
+}
+
+// One group of LPB lines per block; with LOOP, a grid of a.max_blocks blocks
+// walks the line groups (the host-memory form, bound by the CPU-GPU link).
+// Two instances because the loop slows the one-pass form down (up to 20%
+// measured for the C2R lines on GB300).
+// Minimum resident blocks in the launch bounds of the R2C z kernel: 1 (an
+// explicit floor, which changes the compiler's register budget) for float
+// lines of 3 * 2^k >= 384 points, else 0 (no floor).  Measured on GB300 the
+// floor cuts registers 127 -> 107 (M = 768) and 123 -> 95 (M = 384), and
+// the pass time by 7-8% (1536^3: 5.77 -> 5.33 ms); for M = 96 it is 1%
+// slower, and for the C2R kernel, or powers of two, it raises registers.
+template <typename R, int M, int E> __host__ __device__ constexpr int zr2c_minb()
+{
+    return sizeof(R) == 4 && E == 24 && M >= 384 ? 1 : 0;
+}
+
+template <typename R, int M, int E, int LPB, bool LOOP>
+__global__ void __launch_bounds__(LPB *(M / E), zr2c_minb<R, M, E>())
+zpass_r2c_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
+                 const typename twvec<R>::T *__restrict__ rot)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if constexpr (LOOP) {
+        for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
+            if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
+            zr2c_group<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
+        }
+    } else {
+        zr2c_group<R, M, E, LPB, z_l2pf<R, M, false>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+    }
+}
+
+template <typename R, int M, int E, int LPB, bool LOOP>
+__global__ void __launch_bounds__(LPB *(M / E))
+zpass_c2r_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
+                 const typename twvec<R>::T *__restrict__ rot)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if constexpr (LOOP) {
+        for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
+            if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
+            zc2r_group<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
+        }
+    } else {
+        zc2r_group<R, M, E, LPB, z_l2pf<R, M, true>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+    }
+}
+
+// ------------------------------------------------------------ twiddles
+// Stage table of a line plan: entry (m - 1) * ns + k = exp(-2 pi i m k / (ns r)),
+// computed in FP64 with sincospi after exact integer reduction of m k, then
+// rounded once to the storage type.
+template <typename R>
+__global__ void twiddle_stage_kernel(typename cvec<R>::T *out, int ns, int r)
+{
+    typedef typename cvec<R>::T C;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (r - 1) * ns) return;
+    const int m = i / ns + 1;
+    const int k = i - (m - 1) * ns;
+    const int64_t d = (int64_t)ns * r;
+    const int64_t p = ((int64_t)m * k) % d;
+    double s, c;
+    sincospi(2.0 * (double)p / (double)d, &s, &c);
+    out[i] = cmake<C>(R(c), R(-s));
+}
+
+// Fixed-point forms of the two tables, for double lines: entries of scale
+// fx_stage_shift(r), rot[k] of scale kFxRotShift.
+template <typename TW> __global__ void twiddle_stage_fx_kernel(TW *out, int ns, int r)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (r - 1) * ns) return;
+    const int m = i / ns + 1;
+    const int k = i - (m - 1) * ns;
+    const uint32_t d = (uint32_t)ns * (uint32_t)r;
+    out[i] = fx_twiddle((uint32_t)(m * k) % d, d, fx_stage_shift(r));
+}
+template <typename TW> __global__ void twiddle_rot_fx_kernel(TW *out, int n, int count)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < count) out[k] = fx_twiddle((uint32_t)k, (uint32_t)n, kFxRotShift);
+}
+
+// rot[k] = exp(-2 pi i k / n), k < count (FP64 sincospi, rounded once)
+template <typename R>
+__global__ void twiddle_rot_kernel(typename cvec<R>::T *out, int n, int count)
+{
+    typedef typename cvec<R>::T C;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= count) return;
+    double s, c;
+    sincospi(2.0 * (double)k / (double)n, &s, &c);
+    out[k] = cmake<C>(R(c), R(-s));
+}
+
+}  // namespace fft3d

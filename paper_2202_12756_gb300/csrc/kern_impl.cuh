@@ -21,12 +21,11 @@ namespace fft3d {
 
 // Block-size cap of a one-tile-per-block column pass: 1024 threads for float
 // (so a tile row stays one 128-byte segment even at 24 elements per thread,
-// at the price of a few spilled registers there), 256 for double.  Double
-// passes are bound by FP64 issue, not by HBM, so narrower tiles (64-byte row
-// segments of 4 columns at 1024 points) cost them nothing in DRAM terms and
-// let two blocks share an SM, which hides each tile's loads and barriers:
-// measured on GB300 at 1024^3, FP64 column passes 31.5-32.0 -> 30.2-30.3 ms
-// (a 128-thread cap: 30.2 ms; 512 threads, one block per SM: the former).
+// at the price of a few spilled registers there), 256 for double: at 128
+// registers a thread two such blocks share an SM, so that one loads, stores or
+// waits at a barrier while the other computes.  Measured on GB300 at 1024^3
+// (4-column tiles, 64-byte row segments): column passes 6.7 ms, against 8.4-8.7
+// with one block of 512 threads and 8-column tiles.
 template <typename R, int L> __host__ __device__ constexpr int col_max_threads()
 {
     return sizeof(R) == 4 ? FFT3D_COL_MAXT_F32 : (line_E(L) <= 16 ? FFT3D_COL_MAXT_F64 : 256);
@@ -79,10 +78,8 @@ __host__ __device__ constexpr bool pair_axis(int axis) { return axis >= 0 && ((F
 constexpr int kPairW = 16;  // columns of a CTA-pair tile (128-byte float rows)
 
 // Elements per thread of a column pass: 32 in the pipelined kernel, else the
-// default plan of the length; double columns of 512 points, bound by FP64
-// issue, take 8 (radix 8 x 8 x 8: about 28 FP64 operations per point
-// against 28.75 for 16 x 16 x 2; measured at 512^3 the FP64 column passes
-// 3.43 -> 3.34 ms, on 4-column tiles).
+// default plan of the length; double columns of 512 points take 8 (radix 8 x 8
+// x 8, fewer twiddle products than 16 x 16 x 2, on 4-column tiles).
 template <typename R, int L> __host__ __device__ constexpr int col_E()
 {
     return col_pipe<R, L>() ? 32 : ((sizeof(R) == 8 && L == 512) ? 8 : line_E(L));
@@ -98,6 +95,7 @@ template <typename R, int L> __host__ __device__ constexpr int col_W()
         while (w > 1 && w * (L / 32) > 512) w /= 2;
         return w;
     }
+    if (col_fixed<R, L>() && L / col_E<R, L>() < 8) w = 32;  // at least a warp per block
     while (w > 1 && (w * (L / col_E<R, L>()) > col_max_threads<R, L>() ||
                      (size_t)L * w * sizeof(typename cvec<R>::T) > 200 * 1024))
         w /= 2;
@@ -137,7 +135,7 @@ template <typename R, int L> inline void col_geom_t(PassGeom *g, int axis)
     else if (xstage)
         g->smem = xstage_smem_bytes<R, L, E, W>();
     else
-        g->smem = (size_t)L * W * sizeof(C);
+        g->smem = (size_t)L * W * sizeof(C) + (col_fixed<R, L>() ? W * sizeof(int) : 0);  // and the scale codes
 }
 
 template <typename R, int M> inline void z_geom_t(PassGeom *g)
@@ -152,6 +150,13 @@ template <typename R, int M> inline void z_geom_t(PassGeom *g)
     g->smem = (z_paired<R, M>() ? (size_t)(LPB / 2) * zline_smem_elems<2 * M, z_E<R, M>()>()
                                 : (size_t)LPB * zline_smem_elems<M, z_E<R, M>()>()) *
               sizeof(typename cvec<R>::T);
+}
+
+// The kernel that runs one column tile per block.
+template <typename R, int L, bool INV> inline auto col_one_tile_kernel()
+{
+    if constexpr (col_fixed<R, L>()) return colpass_fx_kernel<L, col_E<R, L>(), col_W<R, L>(), INV>;
+    else return colpass_kernel<R, L, col_E<R, L>(), col_W<R, L>(), INV>;
 }
 
 template <typename R, int L> inline cudaError_t col_prepare_t()
@@ -193,11 +198,11 @@ template <typename R, int L> inline cudaError_t col_prepare_t()
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, xs);
             if (e != cudaSuccess) return e;
         }
-        e = cudaFuncSetAttribute(colpass_kernel<R, L, col_E<R, L>(), col_W<R, L>(), false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+        e = cudaFuncSetAttribute(col_one_tile_kernel<R, L, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)g.smem);
         if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(colpass_kernel<R, L, col_E<R, L>(), col_W<R, L>(), true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+        return cudaFuncSetAttribute(col_one_tile_kernel<R, L, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)g.smem);
     }
 }
 
@@ -312,7 +317,7 @@ inline cudaError_t col_launch_t(const ColArgs &a, int64_t tiles, const void *tw,
 {
     PassGeom g;
     col_geom_t<R, L>(&g, a.axis);
-    typedef const typename cvec<R>::T *TW;
+    typedef const typename twvec<R>::T *TW;
     if constexpr (col_pair<R, L>()) {
         if (g.pair) {
             constexpr int E = pair_E<L>(), W = kPairW;
@@ -359,8 +364,7 @@ inline cudaError_t col_launch_t(const ColArgs &a, int64_t tiles, const void *tw,
                 return cudaGetLastError();
             }
         }
-        auto k = a.inverse ? colpass_kernel<R, L, col_E<R, L>(), col_W<R, L>(), true>
-                           : colpass_kernel<R, L, col_E<R, L>(), col_W<R, L>(), false>;
+        auto k = a.inverse ? col_one_tile_kernel<R, L, true>() : col_one_tile_kernel<R, L, false>();
         ColArgs b = a;
         b.pf_stride = col_l2_prefetch<R, L>(a.axis) ? persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) : 0;
         k<<<(unsigned)tiles, g.threads, g.smem, st>>>(b, (TW)tw);
@@ -375,7 +379,7 @@ inline cudaError_t zr2c_launch_t(const ZArgs &a, const void *tw, const void *rot
     z_geom_t<R, M>(&g);
     constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
     const int64_t blocks = (a.nlines + g.per_block - 1) / g.per_block;
-    typedef const typename cvec<R>::T *TW;
+    typedef const typename twvec<R>::T *TW;
     if (a.max_blocks > 0 && blocks > a.max_blocks)
         zpass_r2c_kernel<R, M, E, LPB, true><<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
     else {
@@ -394,7 +398,7 @@ inline cudaError_t zc2r_launch_t(const ZArgs &a, const void *tw, const void *rot
     z_geom_t<R, M>(&g);
     constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
     const int64_t blocks = (a.nlines + g.per_block - 1) / g.per_block;
-    typedef const typename cvec<R>::T *TW;
+    typedef const typename twvec<R>::T *TW;
     if (a.max_blocks > 0 && blocks > a.max_blocks)
         zpass_c2r_kernel<R, M, E, LPB, true><<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
     else {
@@ -445,7 +449,7 @@ inline cudaError_t fused_launch_t(const FusedArgs &a, const void *tw_y, const vo
                                   cudaStream_t st)
 {
     typedef FusedShape<N1, M> S;
-    typedef const typename cvec<R>::T *TW;
+    typedef const typename twvec<R>::T *TW;
     PassGeom g;
     int zl;
     fused_geom_t<R, N1, M>(&g, &zl);
@@ -516,22 +520,21 @@ inline cudaError_t fused_launch_t(const FusedArgs &a, const void *tw_y, const vo
     {                                                                                           \
         const int n = (r - 1) * ns;                                                             \
         if (n <= 0) return cudaSuccess;                                                         \
-        twiddle_stage_kernel<R><<<(n + 255) / 256, 256, 0, st>>>(                              \
-            (typename cvec<R>::T *)out, ns, r);                                                 \
+        if constexpr (sizeof(R) == 8)                                                          \
+            twiddle_stage_fx_kernel<<<(n + 255) / 256, 256, 0, st>>>((fxtw *)out, ns, r);       \
+        else                                                                                    \
+            twiddle_stage_kernel<R><<<(n + 255) / 256, 256, 0, st>>>(                          \
+                (typename cvec<R>::T *)out, ns, r);                                             \
         return cudaGetLastError();                                                              \
     }                                                                                           \
     cudaError_t twiddle_rot_launch_##SUF(void *out, int n, int count, cudaStream_t st)         \
     {                                                                                           \
         if (count <= 0) return cudaSuccess;                                                     \
-        twiddle_rot_kernel<R><<<(count + 255) / 256, 256, 0, st>>>(                            \
-            (typename cvec<R>::T *)out, n, count);                                              \
-        return cudaGetLastError();                                                              \
-    }                                                                                           \
-    cudaError_t twiddle_herm_launch_##SUF(void *out, int n, int count, cudaStream_t st)        \
-    {                                                                                           \
-        if (count <= 0) return cudaSuccess;                                                     \
-        twiddle_herm_kernel<R><<<(count + 255) / 256, 256, 0, st>>>(                           \
-            (typename cvec<R>::T *)out, n, count);                                              \
+        if constexpr (sizeof(R) == 8)                                                          \
+            twiddle_rot_fx_kernel<<<(count + 255) / 256, 256, 0, st>>>((fxtw *)out, n, count);  \
+        else                                                                                    \
+            twiddle_rot_kernel<R><<<(count + 255) / 256, 256, 0, st>>>(                        \
+                (typename cvec<R>::T *)out, n, count);                                          \
         return cudaGetLastError();                                                              \
     }                                                                                           \
     }

@@ -51,14 +51,14 @@ inline int col_table_elems(int L, const PassGeom &g)
     cudaError_t zc2r_launch_##SUF(int M, const ZArgs &a, const void *tw, const void *rot,           \
                                   cudaStream_t st);                                                  \
     cudaError_t twiddle_stage_launch_##SUF(void *out, int ns, int r, cudaStream_t st);             \
-    cudaError_t twiddle_rot_launch_##SUF(void *out, int n, int count, cudaStream_t st);             \
-    cudaError_t twiddle_herm_launch_##SUF(void *out, int n, int count, cudaStream_t st);
+    cudaError_t twiddle_rot_launch_##SUF(void *out, int n, int count, cudaStream_t st);
 
 FFT3D_DECLARE_LAUNCHERS(f32, float)
 FFT3D_DECLARE_LAUNCHERS(f64, double)
 
 // Writes the stage twiddles of an L-point line plan with E elements per
-// thread (FP64 sincospi, rounded once) to dst, on stream st.
+// thread to dst, on stream st: float entries by FP64 sincospi, rounded once;
+// for double lines the fixed-point entries that their transforms multiply by.
 inline cudaError_t write_line_tables(bool f32, int L, int E, void *dst, cudaStream_t st)
 {
     for (int s = 1; s < line_nstages(L, E); ++s) {
@@ -86,13 +86,11 @@ inline cudaError_t write_col_tables(bool f32, int L, const PassGeom &g, void *ds
 inline int z_line_points(int m, const PassGeom &gz) { return gz.pair ? 2 * m : m; }
 
 // Table of the contiguous-axis passes of an N2 = 2M point line (`rot` of
-// the z launchers): float lines take the R2C rotations exp(-2 pi i k / N2),
-// k < M; double lines take the [A, B] coefficient pairs of their Hermitian
-// post- / pre-process for k <= M (see twiddle_herm_kernel).
-inline size_t z_table_elems(bool f32, int m) { return f32 ? (size_t)m : 2 * ((size_t)m + 1); }
+// the z launchers): the R2C rotations exp(-2 pi i k / N2), k < M.
+inline size_t z_table_elems(int m) { return (size_t)m; }
 inline cudaError_t write_z_table(bool f32, int n2, void *dst, cudaStream_t st)
 {
-    return f32 ? twiddle_rot_launch_f32(dst, n2, n2 / 2, st) : twiddle_herm_launch_f64(dst, n2, n2 / 2 + 1, st);
+    return f32 ? twiddle_rot_launch_f32(dst, n2, n2 / 2, st) : twiddle_rot_launch_f64(dst, n2, n2 / 2, st);
 }
 
 // Fused plane pass (float only): available for (N1, M) in

@@ -1,5 +1,6 @@
-// Register-resident Stockham line FFT: complex helpers, radix-2/3/4/8/16
-// butterflies and the stage engine used by every pass kernel.
+// Register-resident Stockham line FFT: complex helpers, radix-2/3/4/8/16/24/32
+// butterflies and the stage engine used by every pass kernel, for float,
+// double and the fixed-point numbers of fx_math.cuh.
 //
 // All butterflies compute the forward DFT y[k] = sum_n a[n] exp(-2 pi i n k / R)
 // (Eq. 1's sign).  Inverse transforms reuse them through
@@ -10,6 +11,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
+#include "fx_math.cuh"
 #include "line_plan.cuh"
 
 namespace fft3d {
@@ -17,6 +21,13 @@ namespace fft3d {
 template <typename R> struct cvec;
 template <> struct cvec<float> { typedef float2 T; };
 template <> struct cvec<double> { typedef double2 T; };
+template <> struct cvec<fx64> { typedef fxc T; };
+// twiddle table entries: rounded once to float for float lines; double lines
+// are transformed in fixed point, and their FP64 path (for the few lines that
+// need it) reads the same table
+template <typename R> struct twvec { typedef typename cvec<R>::T T; };
+template <> struct twvec<double> { typedef fxtw T; };
+template <> struct twvec<fx64> { typedef fxtw T; };
 
 template <typename C> __device__ __forceinline__ C cmake(decltype(C::x) x, decltype(C::x) y)
 {
@@ -79,6 +90,21 @@ template <typename C> struct Dft<3, C> {
     }
 };
 
+// fixed point: the half sum is rounded, the rotation is one of 90 degrees
+// after a scaling by sin 60 = cos 30 degrees
+template <> struct Dft<3, fxc> {
+    __device__ __forceinline__ static void run(fxc *a)
+    {
+        const fxc t = cadd(a[1], a[2]);
+        const fxc u = csub(a[1], a[2]);
+        const fxc m = fx_make(a[0].x - ((t.x + 1) >> 1), a[0].y - ((t.y + 1) >> 1));
+        const fxc v = fx_make(fx_scale96<8>(u.y), -fx_scale96<8>(u.x));
+        a[0] = cadd(a[0], t);
+        a[1] = cadd(m, v);
+        a[2] = csub(m, v);
+    }
+};
+
 template <typename C> __device__ __forceinline__ void dft4(C &a0, C &a1, C &a2, C &a3)
 {
     const C t0 = cadd(a0, a2);
@@ -130,29 +156,39 @@ template <typename C> struct Dft<8, C> {
     }
 };
 
+// z * exp(-2 pi i P / 16), P = 1, 3 or 9
+template <int P, typename C> __device__ __forceinline__ C w16(C z)
+{
+    static_assert(P == 1 || P == 3 || P == 9, "the radix-16 butterfly's general rotations");
+    if constexpr (std::is_same<C, fxc>::value) {
+        return fx_rot96<6 * P>(z);
+    } else {
+        typedef decltype(C::x) R;
+        constexpr double c = P == 1 ? FFT3D_C8 : (P == 3 ? FFT3D_S8 : -FFT3D_C8);
+        constexpr double s = P == 1 ? -FFT3D_S8 : (P == 3 ? -FFT3D_C8 : FFT3D_S8);
+        return cmul(z, cmake<C>(R(c), R(s)));
+    }
+}
+
 template <typename C> struct Dft<16, C> {
     // radix 4 x 4: n = 4 n1 + n2, k = k1 + 4 k2;
     // y[k1 + 4 k2] = sum_{n2} W16^{n2 k1} W4^{n2 k2} sum_{n1} a[4 n1 + n2] W4^{n1 k1}
     __device__ __forceinline__ static void run(C *a)
     {
-        typedef decltype(C::x) R;
         dft4(a[0], a[4], a[8], a[12]);
         dft4(a[1], a[5], a[9], a[13]);
         dft4(a[2], a[6], a[10], a[14]);
         dft4(a[3], a[7], a[11], a[15]);
         // a[n2 + 4 k1] now holds the inner sum for (n2, k1); twiddle by W16^{n2 k1}
-        const C w1 = cmake<C>(R(FFT3D_C8), -R(FFT3D_S8));
-        const C w3 = cmake<C>(R(FFT3D_S8), -R(FFT3D_C8));
-        const C w9 = cmake<C>(-R(FFT3D_C8), R(FFT3D_S8));
-        a[5] = cmul(a[5], w1);     // n2=1, k1=1
+        a[5] = w16<1>(a[5]);       // n2=1, k1=1
         a[9] = w8_1(a[9]);         // n2=1, k1=2 : W16^2
-        a[13] = cmul(a[13], w3);   // n2=1, k1=3
+        a[13] = w16<3>(a[13]);     // n2=1, k1=3
         a[6] = w8_1(a[6]);         // n2=2, k1=1 : W16^2
         a[10] = cmul_mi(a[10]);    // n2=2, k1=2 : W16^4
         a[14] = w8_3(a[14]);       // n2=2, k1=3 : W16^6
-        a[7] = cmul(a[7], w3);     // n2=3, k1=1
+        a[7] = w16<3>(a[7]);       // n2=3, k1=1
         a[11] = w8_3(a[11]);       // n2=3, k1=2 : W16^6
-        a[15] = cmul(a[15], w9);   // n2=3, k1=3
+        a[15] = w16<9>(a[15]);     // n2=3, k1=3
         dft4(a[0], a[1], a[2], a[3]);
         dft4(a[4], a[5], a[6], a[7]);
         dft4(a[8], a[9], a[10], a[11]);
@@ -222,7 +258,9 @@ template <typename C> struct Dft<32, C> {
 template <int P, typename C> __device__ __forceinline__ C w24(C z)
 {
     constexpr int p = P % 24;
-    if constexpr (p == 0) {
+    if constexpr (std::is_same<C, fxc>::value) {
+        return fx_rot96<4 * p>(z);
+    } else if constexpr (p == 0) {
         return z;
     } else if constexpr (p == 3) {
         return w8_1(z);
@@ -289,8 +327,22 @@ template <typename C> struct Dft<24, C> {
 // copied to shared memory (TWS).
 template <bool TWS, typename C> __device__ __forceinline__ C tw_read(const C *__restrict__ tw, int i)
 {
-    if constexpr (TWS) return tw[i];
-    else return __ldg(tw + i);
+    if constexpr (TWS) {
+        return tw[i];
+    } else if constexpr (std::is_same<C, fxtw>::value) {
+        const int4 q = __ldg((const int4 *)(tw + i));
+        return fxtw{q.x, q.y, q.z, q.w};
+    } else {
+        return __ldg(tw + i);
+    }
+}
+// t times a table twiddle of scale D: fixed-point values are scaled by 2^-D,
+// double values by the factor itself.
+template <int D> __device__ __forceinline__ float2 tw_mul(float2 t, float2 w) { return cmul(t, w); }
+template <int D> __device__ __forceinline__ fxc tw_mul(fxc t, fxtw w) { return cmul(t, w); }
+template <int D> __device__ __forceinline__ double2 tw_mul(double2 t, fxtw w)
+{
+    return cmul(t, cmake<double2>(fx_twiddle_value(w.xh, w.xl, D), fx_twiddle_value(w.yh, w.yl, D)));
 }
 
 // Compile-time loop: f(IntC<I>()) for I = B .. N-1.
@@ -311,7 +363,7 @@ template <int B, int N, class F> __device__ __forceinline__ void static_for(cons
 
 template <typename R, int L, int E, int S, bool TWS = false>
 __device__ __forceinline__ void line_stage_compute(typename cvec<R>::T *v, int j,
-                                                   const typename cvec<R>::T *__restrict__ tw)
+                                                   const typename twvec<R>::T *__restrict__ tw)
 {
     typedef typename cvec<R>::T C;
     constexpr int NT = L / E;
@@ -354,9 +406,11 @@ __device__ __forceinline__ void line_stage_compute(typename cvec<R>::T *v, int j
             C t[RS];
 #pragma unroll
             for (int m = 0; m < RS; ++m) t[m] = v[q + m * Q];
-            if (S > 0) {
+            if constexpr (S > 0) {
+                constexpr int D = fx_stage_shift(RS);
+                if constexpr (std::is_same<R, fx64>::value) t[0] = fx_shr<D>(t[0]);
 #pragma unroll
-                for (int m = 1; m < RS; ++m) t[m] = cmul(t[m], tw_read<TWS>(tw, TWO + (m - 1) * NS + k));
+                for (int m = 1; m < RS; ++m) t[m] = tw_mul<D>(t[m], tw_read<TWS>(tw, TWO + (m - 1) * NS + k));
             }
             Dft<RS, C>::run(t);
 #pragma unroll
@@ -444,7 +498,7 @@ __device__ __forceinline__ void line_exchange(typename cvec<R>::T *v, int j, Ex 
 
 template <typename R, int L, int E, int S, bool TWS, class Ex, class Hook, class Tail>
 __device__ __forceinline__ void line_stages_from(typename cvec<R>::T *v, int j,
-                                                 const typename cvec<R>::T *__restrict__ tw, Ex &ex,
+                                                 const typename twvec<R>::T *__restrict__ tw, Ex &ex,
                                                  const Hook &hook, const Tail &tail)
 {
     if constexpr (S < line_nstages(L, E)) {
@@ -461,6 +515,13 @@ __device__ __forceinline__ void line_stages_from(typename cvec<R>::T *v, int j,
     }
 }
 
+// Power of two by which a fixed-point transform scales its result down.
+template <int L, int E, int S = 1> __host__ __device__ constexpr int fx_line_shift()
+{
+    if constexpr (S < line_nstages(L, E)) return fx_stage_shift(line_radix(L, E, S)) + fx_line_shift<L, E, S + 1>();
+    else return 0;
+}
+
 // Forward FFT of a line held as v[i] = x[j + i NT]; result in the same slots.
 // `hook` runs once after the first exchange barrier (or after the only
 // stage); `tail` runs once after the last exchange has ended on a barrier, so
@@ -469,7 +530,7 @@ __device__ __forceinline__ void line_stages_from(typename cvec<R>::T *v, int j,
 // memory.
 template <typename R, int L, int E, bool TWS = false, class Ex, class Hook = NoHook, class Tail = NoHook>
 __device__ __forceinline__ void line_fft(typename cvec<R>::T *v, int j,
-                                         const typename cvec<R>::T *__restrict__ tw, Ex &ex,
+                                         const typename twvec<R>::T *__restrict__ tw, Ex &ex,
                                          const Hook &hook = Hook(), const Tail &tail = Tail())
 {
     static_assert(line_plan_valid(L, E), "invalid line plan");

@@ -7,7 +7,8 @@
 //               E = (Z[k] + conj Z[M-k]) / 2, O = (Z[k] - conj Z[M-k]) / 2i.
 //               (Step 1 of Sec. 3 along the first of the two plane axes.)
 //               Double lines of N2 = 1024 points instead run two lines per
-//               N2-point complex transform (zr2c_pairs / zc2r_pairs).
+//               N2-point complex transform (zr2c_pairs / zc2r_pairs).  The
+//               double forms here are the slow path of fx_kernels.cuh.
 //   zpass_c2r : inverse, contiguous axis 2: the same relation run backwards,
 //               then the M-point inverse FFT, the unpacking into 2M reals and
 //               the 1/(N0 N1 N2) normalisation (the paper's separate
@@ -169,7 +170,7 @@ template <typename C> __device__ __forceinline__ C load_cg(const C *p) { return 
 // loaded straight into registers.  CG selects L2-only loads.
 template <typename R, int L, int E, int W, bool CG, bool INV>
 __device__ __forceinline__ void col_tile(const ColArgs &a, int64_t tile, unsigned char *smem,
-                                         const typename cvec<R>::T *__restrict__ tw, int64_t pf_tile = -1)
+                                         const typename twvec<R>::T *__restrict__ tw, int64_t pf_tile = -1)
 {
     typedef typename cvec<R>::T C;
     constexpr int NT = L / E;
@@ -214,7 +215,7 @@ __device__ __forceinline__ void col_tile(const ColArgs &a, int64_t tile, unsigne
 // One tile per block.
 template <typename R, int L, int E, int W, bool INV>
 __global__ void __launch_bounds__(W *(L / E))
-colpass_kernel(ColArgs a, const typename cvec<R>::T *__restrict__ tw)
+colpass_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int64_t pf = a.pf_stride > 0 && blockIdx.x + a.pf_stride < gridDim.x ? blockIdx.x + a.pf_stride : -1;
@@ -331,7 +332,7 @@ template <typename R, int L, int E, int W> __host__ __device__ constexpr size_t 
 // (stores interleaved with the next tile's staging reads) by 9-25%.
 template <typename R, int L, int E, int W, bool INV, bool EARLY>
 __global__ void __launch_bounds__(W *(L / E), (W * (L / E) >= 512 ? 1 : 512 / (W * (L / E))))
-colpass_pipe_kernel(ColArgs a, const typename cvec<R>::T *__restrict__ tw, int64_t ntiles,
+colpass_pipe_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int64_t ntiles,
                     const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap2)
 {
     typedef typename cvec<R>::T C;
@@ -513,7 +514,7 @@ template <typename R, int L, int E, int W> __host__ __device__ constexpr size_t 
 
 template <typename R, int L, int E, int W, bool INV>
 __global__ void __launch_bounds__(W *(L / E), 1)
-colpass_xstage_kernel(ColArgs a, const typename cvec<R>::T *__restrict__ tw, int64_t ntiles,
+colpass_xstage_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int64_t ntiles,
                     const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap2)
 {
     typedef typename cvec<R>::T C;
@@ -778,7 +779,7 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint32_t mb, uint32_t 
 
 template <typename R, int L, int E, int W, bool INV, bool EARLY>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(W *(L / 2 / E), 1)
-colpass_pair_kernel(ColArgs a, const typename cvec<R>::T *__restrict__ tw, int64_t ntiles,
+colpass_pair_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int64_t ntiles,
                     const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap2)
 {
     typedef typename cvec<R>::T C;
@@ -1008,11 +1009,9 @@ struct ZArgs {
 // of a thread; measured on GB300 it halves the resident warps and runs 25%
 // slower at M = 512, and at M = 1024 (150-170 registers, one block per SM)
 // 45% slower.
-// Double lines of N2 = 1024 points (M = 512), bound by FP64 issue, run two
-// lines per complex transform of N2 points (z_paired, zr2c_pairs /
-// zc2r_pairs below; 16 elements per thread, radix 16 x 16 x 4): about 33.9
-// FP64 operations per element against 36.4 for the half-length scheme on
-// radix 8 x 8 x 8; measured at 1024^3 the FP64 z-passes 36.1 -> 34.5 ms.
+// Double lines of N2 = 1024 points (M = 512) run two lines per complex
+// transform of N2 points (z_paired; 16 elements per thread, radix 16 x 16 x 4):
+// no Hermitian rotation, one twiddle product per element fewer.
 template <typename R, int M> __host__ __device__ constexpr bool z_paired() { return sizeof(R) == 8 && M == 512; }
 template <typename R, int M> __host__ __device__ constexpr int z_E() { return z_paired<R, M>() ? 16 : line_E(M); }
 
@@ -1078,7 +1077,7 @@ template <typename R, int M, bool C2R> __host__ __device__ constexpr bool z_l2pf
 // exp(-i pi i / E) (NT / 2M = 1 / 2E); double lines load every factor.
 template <typename R, int E, int I>
 __device__ __forceinline__ typename cvec<R>::T z_rot(typename cvec<R>::T rot_j,
-                                                     const typename cvec<R>::T *__restrict__ rot, int k)
+                                                     const typename twvec<R>::T *__restrict__ rot, int k)
 {
     typedef typename cvec<R>::T C;
     if constexpr (FFT3D_ROTCONST && sizeof(R) == 4) {
@@ -1088,6 +1087,8 @@ __device__ __forceinline__ typename cvec<R>::T z_rot(typename cvec<R>::T rot_j,
             constexpr CtCosSin w = ct_cossin_pi(-(long long)I, E);
             return cmul(rot_j, cmake<C>(R(w.c), R(w.s)));
         }
+    } else if constexpr (sizeof(R) == 8) {
+        return cmake<C>(fx_twiddle_value(rot[k].xh, rot[k].xl, 2), fx_twiddle_value(rot[k].yh, rot[k].yl, 2));
     } else {
         return __ldg(rot + k);
     }
@@ -1098,12 +1099,11 @@ __device__ __forceinline__ typename cvec<R>::T z_rot(typename cvec<R>::T rot_j,
 // Thread j holds Z[j + i NT]; the partner Z[M - k] of k = j + i NT is slot
 // E - 1 - i of lane NT - j (j > 0) or this lane's slot (E - i) mod E (j = 0),
 // so when a float line fits a warp the post-process takes it by shuffle
-// (double lines, bound by FP64 arithmetic, keep the shared-memory exchange
-// and its lower register count).
+// (double lines keep the shared-memory exchange and its lower register count).
 template <typename R, int M, int E, int LPB, bool PF = false>
 __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsigned char *smem,
-                                           const typename cvec<R>::T *__restrict__ tw,
-                                           const typename cvec<R>::T *__restrict__ rot)
+                                           const typename twvec<R>::T *__restrict__ tw,
+                                           const typename twvec<R>::T *__restrict__ rot)
 {
     typedef typename cvec<R>::T C;
     constexpr int NT = M / E;
@@ -1150,10 +1150,8 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
             emit(k, v[i], zm, z_rot<R, E, i>(rot_j, rot, k));
         });
     } else if constexpr (sizeof(R) == 8) {
-        // Double lines (bound by FP64 issue): X[k] = A[k] Z[k] + B[k] conj(Z[M - k]),
-        // A = (1 - i r) / 2, B = (1 + i r) / 2 from the coefficient table (`rot`
-        // holds [A, B] pairs), 8 FP64 operations per element instead of 12; the
-        // output scale is applied only when it is not 1.
+        // Double lines: X[k] = A[k] Z[k] + B[k] conj(Z[M - k]), A = (1 - i r) / 2,
+        // B = (1 + i r) / 2; the output scale is applied only when it is not 1.
         constexpr bool LR = pad_linear_reads<P>(NT);
         constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
 #pragma unroll
@@ -1165,7 +1163,8 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
             const int k = j + i * NT;
             const C z = ex.get(pad_row<P, LR>(j, i * NT));
             const C zm = (i == 0 && j == 0) ? z : ex.get(pad_row<P, LREV>(M - j, -i * NT));
-            const C A = __ldg(rot + 2 * k), B = __ldg(rot + 2 * k + 1);
+            const C r = z_rot<R, E, i>(rot_j, rot, k);
+            const C A = cmake<C>(R(0.5) + R(0.5) * r.y, R(-0.5) * r.x), B = cmake<C>(R(0.5) - R(0.5) * r.y, R(0.5) * r.x);
             // A z + B conj(zm)
             C x = cmake<C>(fma(A.x, z.x, fma(-A.y, z.y, fma(B.x, zm.x, B.y * zm.y))),
                            fma(A.x, z.y, fma(A.y, z.x, fma(B.y, zm.x, -B.x * zm.y))));
@@ -1198,8 +1197,8 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
 // with X[M], which it loads itself).
 template <typename R, int M, int E, int LPB, bool CG, bool PF = false>
 __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsigned char *smem,
-                                           const typename cvec<R>::T *__restrict__ tw,
-                                           const typename cvec<R>::T *__restrict__ rot)
+                                           const typename twvec<R>::T *__restrict__ tw,
+                                           const typename twvec<R>::T *__restrict__ rot)
 {
     typedef typename cvec<R>::T C;
     constexpr int NT = M / E;
@@ -1278,13 +1277,15 @@ __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsign
             C y = ex.get(pad_row<P, LREV>(M - j, -i * NT));  // X[M - k]; k = 0 pairs with X[M]
             if constexpr (sizeof(R) == 8) {
                 // Double lines: conj Z[k] = 2 (A[k] conj(x) + B[k] y) with the
-                // coefficient table of the R2C lines (8 FP64 operations instead
-                // of 10); the factor 2 goes into the output scale below.
+                // coefficients of the R2C lines; the factor 2 goes into the output
+                // scale below.
                 if (k == 0) {
                     x = cmake<C>(we * x.x, R(0));
                     y = cmake<C>(we * y.x, R(0));
                 }
-                const C A = __ldg(rot + 2 * k), B = __ldg(rot + 2 * k + 1);
+                const C r = z_rot<R, E, i>(rot_j, rot, k);
+                const C A = cmake<C>(R(0.5) + R(0.5) * r.y, R(-0.5) * r.x),
+                        B = cmake<C>(R(0.5) - R(0.5) * r.y, R(0.5) * r.x);
                 v[i] = cmake<C>(fma(A.x, x.x, fma(A.y, x.y, fma(B.x, y.x, -B.y * y.y))),
                                 fma(A.y, x.x, fma(-A.x, x.y, fma(B.x, y.y, B.y * y.x))));
             } else {
@@ -1316,7 +1317,7 @@ __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsign
 // odd line count the last pair's second line is zero and not written.
 template <typename R, int M, int E, int LPB>
 __device__ __forceinline__ void zr2c_pairs(const ZArgs &a, int64_t line0, unsigned char *smem,
-                                           const typename cvec<R>::T *__restrict__ tw)
+                                           const typename twvec<R>::T *__restrict__ tw)
 {
     typedef typename cvec<R>::T C;
     constexpr int N = 2 * M;
@@ -1371,7 +1372,7 @@ __device__ __forceinline__ void zr2c_pairs(const ZArgs &a, int64_t line0, unsign
 // with the output scale.  CG selects L2-only loads.
 template <typename R, int M, int E, int LPB, bool CG>
 __device__ __forceinline__ void zc2r_pairs(const ZArgs &a, int64_t line0, unsigned char *smem,
-                                           const typename cvec<R>::T *__restrict__ tw)
+                                           const typename twvec<R>::T *__restrict__ tw)
 {
     typedef typename cvec<R>::T C;
     constexpr int N = 2 * M;
@@ -1431,107 +1432,6 @@ __device__ __forceinline__ void zc2r_pairs(const ZArgs &a, int64_t line0, unsign
         if (act0) store_out(out0 + j + i * NT, s * z.x);
         if (act1) store_out(out1 + j + i * NT, s * z.y);
     }
-}
-
-// One group of LPB lines per block; with LOOP, a grid of a.max_blocks blocks
-// walks the line groups (the host-memory form, bound by the CPU-GPU link).
-// Two instances because the loop slows the one-pass form down (up to 20%
-// measured for the C2R lines on GB300).
-// Minimum resident blocks in the launch bounds of the R2C z kernel: 1 (an
-// explicit floor, which changes the compiler's register budget) for float
-// lines of 3 * 2^k >= 384 points, else 0 (no floor).  Measured on GB300 the
-// floor cuts registers 127 -> 107 (M = 768) and 123 -> 95 (M = 384), and
-// the pass time by 7-8% (1536^3: 5.77 -> 5.33 ms); for M = 96 it is 1%
-// slower, and for the C2R kernel, or powers of two, it raises registers.
-template <typename R, int M, int E> __host__ __device__ constexpr int zr2c_minb()
-{
-    return sizeof(R) == 4 && E == 24 && M >= 384 ? 1 : 0;
-}
-
-template <typename R, int M, int E, int LPB, bool LOOP>
-__global__ void __launch_bounds__(LPB *(M / E), zr2c_minb<R, M, E>())
-zpass_r2c_kernel(ZArgs a, const typename cvec<R>::T *__restrict__ tw,
-                 const typename cvec<R>::T *__restrict__ rot)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    if constexpr (LOOP) {
-        for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
-            if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
-            if constexpr (z_paired<R, M>()) zr2c_pairs<R, M, E, LPB>(a, blk * LPB, smem_raw, tw);
-            else zr2c_lines<R, M, E, LPB>(a, blk * LPB, smem_raw, tw, rot);
-        }
-    } else if constexpr (z_paired<R, M>()) {
-        zr2c_pairs<R, M, E, LPB>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw);
-    } else {
-        zr2c_lines<R, M, E, LPB, z_l2pf<R, M, false>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
-    }
-}
-
-template <typename R, int M, int E, int LPB, bool LOOP>
-__global__ void __launch_bounds__(LPB *(M / E))
-zpass_c2r_kernel(ZArgs a, const typename cvec<R>::T *__restrict__ tw,
-                 const typename cvec<R>::T *__restrict__ rot)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    if constexpr (LOOP) {
-        for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
-            if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
-            if constexpr (z_paired<R, M>()) zc2r_pairs<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw);
-            else zc2r_lines<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
-        }
-    } else if constexpr (z_paired<R, M>()) {
-        zc2r_pairs<R, M, E, LPB, false>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw);
-    } else {
-        zc2r_lines<R, M, E, LPB, false, z_l2pf<R, M, true>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
-    }
-}
-
-// ------------------------------------------------------------ twiddles
-// Stage table of a line plan: entry (m - 1) * ns + k = exp(-2 pi i m k / (ns r)),
-// computed in FP64 with sincospi after exact integer reduction of m k, then
-// rounded once to the storage type.
-template <typename R>
-__global__ void twiddle_stage_kernel(typename cvec<R>::T *out, int ns, int r)
-{
-    typedef typename cvec<R>::T C;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (r - 1) * ns) return;
-    const int m = i / ns + 1;
-    const int k = i - (m - 1) * ns;
-    const int64_t d = (int64_t)ns * r;
-    const int64_t p = ((int64_t)m * k) % d;
-    double s, c;
-    sincospi(2.0 * (double)p / (double)d, &s, &c);
-    out[i] = cmake<C>(R(c), R(-s));
-}
-
-// Coefficients of the Hermitian post- / pre-process of double lines, for
-// k <= count - 1: with r = exp(-2 pi i k / n) = (cos t, -sin t),
-//   out[2k] = A = (1 - i r) / 2 = ((1 - sin t) / 2, -cos t / 2),
-//   out[2k + 1] = B = (1 + i r) / 2 = ((1 + sin t) / 2, cos t / 2),
-// computed in FP64 from sincospi (after exact reduction of k mod n).
-template <typename R>
-__global__ void twiddle_herm_kernel(typename cvec<R>::T *out, int n, int count)
-{
-    typedef typename cvec<R>::T C;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    double s, c;
-    sincospi(2.0 * (double)(k % n) / (double)n, &s, &c);
-    out[2 * k] = cmake<C>(R(0.5 - 0.5 * s), R(-0.5 * c));
-    out[2 * k + 1] = cmake<C>(R(0.5 + 0.5 * s), R(0.5 * c));
-}
-
-// rot[k] = exp(-2 pi i k / n), k < count (FP64 sincospi, rounded once)
-template <typename R>
-__global__ void twiddle_rot_kernel(typename cvec<R>::T *out, int n, int count)
-{
-    typedef typename cvec<R>::T C;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    double s, c;
-    sincospi(2.0 * (double)k / (double)n, &s, &c);
-    out[k] = cmake<C>(R(c), R(-s));
 }
 
 }  // namespace fft3d
