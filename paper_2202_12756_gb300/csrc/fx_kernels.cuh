@@ -522,8 +522,9 @@ __device__ __forceinline__ void zc2r_group(const ZArgs &a, int64_t line0, unsign
 // slower, and for the C2R kernel, or powers of two, it raises registers.
 template <typename R, int M, int E> __host__ __device__ constexpr int zr2c_minb()
 {
-    return sizeof(R) == 4 && E == 24 && M >= 384 ? 1 : 0;
+    return sizeof(R) == 4 ? (E == 24 && M >= 384 ? 1 : 0) : (z_fixed<R, M>() ? 2 : 0);
 }
+template <typename R, int M> __host__ __device__ constexpr int zc2r_minb() { return z_fixed<R, M>() ? 2 : 0; }
 
 template <typename R, int M, int E, int LPB, bool LOOP>
 __global__ void __launch_bounds__(LPB *(M / E), zr2c_minb<R, M, E>())
@@ -542,7 +543,7 @@ zpass_r2c_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__
 }
 
 template <typename R, int M, int E, int LPB, bool LOOP>
-__global__ void __launch_bounds__(LPB *(M / E))
+__global__ void __launch_bounds__(LPB *(M / E), zc2r_minb<R, M>())
 zpass_c2r_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
                  const typename twvec<R>::T *__restrict__ rot)
 {
