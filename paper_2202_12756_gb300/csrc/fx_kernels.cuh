@@ -5,9 +5,8 @@
 // double range) runs the FP64 pass instead, from the same twiddle tables.
 //
 // Measured on GB300 in place (FP64 arithmetic -> fixed point): 1024^3 pair
-// 190.1 -> 43.9 ms (column passes 30.3 -> 6.7 ms each, z-passes 34.5 -> 6.5 and
-// 10.5), 512^3 21.6 -> 5.85 ms; relative L2 error of one transform 2.0-2.6e-16
-// -> 0.8-1.6e-16 against quadruple precision over every line length.
+// 190.1 -> 36 ms, 512^3 21.6 -> 4.1 ms; relative L2 error of one transform
+// 2.0-2.6e-16 -> 0.8-1.6e-16 against quadruple precision over every line length.
 #pragma once
 
 #include "pass_kernels.cuh"
@@ -41,22 +40,71 @@ template <int N> __device__ __forceinline__ int fx_thread_code(const double2 *v)
     return fx_code(tm, s);
 }
 
-// Half of a complex result by the integer pipe, half by the (otherwise idle)
-// FP64 pipe.
-__device__ __forceinline__ double2 fx_out(fxc z, int e) { return cmake<double2>(fx_to(z.x, e), fx_to_fp(z.y, e)); }
+// A complex result: by integer operations, or where a component is below 2^32
+// (2^-29 of the line's scale) or zero, by FP64 additions.
+__device__ __forceinline__ double2 fx_out(fxc z, int e)
+{
+    int32_t big = -1;
+    double2 r = cmake<double2>(fx_to_big(z.x, e, big), fx_to_big(z.y, e, big));
+    if (big >= 0) r = cmake<double2>(fx_to(z.x, e), fx_to(z.y, e));
+    return r;
+}
+// A thread's results v[i] 2^e, handed to f(i, value).  Small components are
+// noticed on the way and all results handed over again by FP64 additions.
+template <int E, class F> __device__ __forceinline__ void fx_out_all(const fxc *v, int e, const F &f)
+{
+    int32_t big = -1;
+#pragma unroll
+    for (int i = 0; i < E; ++i) f(i, cmake<double2>(fx_to_big(v[i].x, e, big), fx_to_big(v[i].y, e, big)));
+    if (big >= 0) {
+        fxc w[E];
+#pragma unroll
+        for (int i = 0; i < E; ++i) w[i] = v[i];
+#pragma unroll 1
+        for (int i = 0; i < E; ++i) f(i, cmake<double2>(fx_to(w[i].x, e), fx_to(w[i].y, e)));
+    }
+}
+
+// z f, or z itself in the UNIT kernels, whose scales are 1 or (C2R) a power of
+// two: a product costs an FP64 issue slot even where it is predicated off.
+template <bool UNIT> __device__ __forceinline__ double2 fx_scale(double2 z, double f)
+{
+    if constexpr (UNIT) return z;
+    else return cscale(z, f);
+}
 
 // ------------------------------------------------------------ columns
+// Load of a column entry, asking L2 for the whole 128-byte line: the tile beside
+// it, run at the same time by another SM, wants the rest of it (512^3: y-pass
+// 0.646 -> 0.636 ms).
+__device__ __forceinline__ double2 fx_load(const double2 *p)
+{
+    double2 r;
+    asm volatile("ld.global.L2::128B.v2.f64 {%0, %1}, [%2];\n" : "=d"(r.x), "=d"(r.y) : "l"(p) : "memory");
+    return r;
+}
+
 template <int L, int E, int W, bool INV>
 __device__ __noinline__ void col_tile_slow(const ColArgs &a, int64_t tile, unsigned char *smem, const fxtw *tw)
 {
     col_tile<double, L, E, W, false, INV>(a, tile, smem, tw);
 }
 
+// Threads that are to share an SM: 64 registers each with 8 elements per
+// thread, 168 with 24 in blocks of 128, else 128.
+__host__ __device__ constexpr int fx_resident(int E, int block) { return E <= 8 ? 1024 : E == 24 && block <= 128 ? 384 : 512; }
+__host__ __device__ constexpr int fx_min_blocks(int E, int block)
+{
+    const int n = fx_resident(E, block) / block;
+    return n < 1 ? 1 : n > 32 ? 32 : n;
+}
+
 template <int L, int E, int W, bool INV>
-__global__ void __launch_bounds__(W *(L / E), (W * (L / E) >= 512 ? 1 : 512 / (W * (L / E))))
+__global__ void __launch_bounds__(W *(L / E), fx_min_blocks(E, W *(L / E)))
 colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw)
 {
     constexpr int NT = L / E;
+    static_assert(W <= 32 && W * NT % 32 == 0, "a warp holds all columns of the tile");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int *code = (int *)(smem_raw + (size_t)L * W * sizeof(fxc));
     const int c = threadIdx.x % W;
@@ -72,7 +120,7 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
         const double2 *sj = sp + (int64_t)j * ss;
         const int64_t sstep = (int64_t)NT * ss;
 #pragma unroll
-        for (int i = 0; i < E; ++i) r[i] = sj[i * sstep];
+        for (int i = 0; i < E; ++i) r[i] = fx_load(sj + i * sstep);
         if constexpr (NT > 1) {
             g = fx_thread_code<E>(r);
             __syncthreads();
@@ -88,15 +136,12 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
             code[c] = g;
         }
         __syncthreads();
-        bool ok = true;
-#pragma unroll
-        for (int i = 0; i < W; ++i) ok = ok && fx_code_ok(code[i]);
-        if (!ok) {
+        g = code[c];
+        if (!__all_sync(0xffffffffu, fx_code_ok(g))) {  // every warp holds every column of the tile
             __syncthreads();
             col_tile_slow<L, E, W, INV>(a, blockIdx.x, smem_raw, tw);
             return;
         }
-        g = code[c];
         g = g == 0 ? kFxZeroCode : g;
 #pragma unroll
         for (int i = 0; i < E; ++i)
@@ -108,12 +153,7 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
     if (valid) {
         double2 *dj = dp + (int64_t)j * ds;
         const int64_t dstep = (int64_t)NT * ds;
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            double2 o = fx_out(v[i], e);
-            if (INV) o = cswap(o);
-            dj[i * dstep] = o;
-        }
+        fx_out_all<E>(v, e, [&](int i, double2 o) { dj[i * dstep] = INV ? cswap(o) : o; });
     }
 }
 
@@ -158,7 +198,7 @@ __device__ __noinline__ void zc2r_slow(const ZArgs &a, int64_t line0, unsigned c
 
 // zr2c_lines in fixed point: X[k] = (s - i r d) / 2 with s = Z[k] + conj Z[M - k],
 // d = Z[k] - conj Z[M - k], formed as X / 2 = s / 4 - i (r / 4) d.
-template <int M, int E, int LPB>
+template <int M, int E, int LPB, bool UNIT>
 __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, unsigned char *smem,
                                               const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
 {
@@ -191,14 +231,12 @@ __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, uns
     const int e = g - 1023 - kFxBits + fx_line_shift<M, E>();
     double2 *out = (double2 *)a.cplx.main + (active ? line : 0) * (M + 1);
     const double se = a.scale_edge, sm = a.scale_mid;
-    const bool unit = se == 1.0 && sm == 1.0;
     auto emit = [&](int k, fxc z, fxc zm) {
         const fxc zc = cconj(zm);
         const fxc s = fx_shr<2>(cadd(z, zc));
         const fxc p = cmul(csub(z, zc), fx_ldg(rot + k));
-        double2 x = fx_out(fx_make(s.x + p.y, s.y - p.x), e + 1);
-        if (!unit) x = cscale(x, k == 0 ? se : sm);
-        if (active) store_out(out + k, x);
+        const double2 x = fx_out(fx_make(s.x + p.y, s.y - p.x), e + 1);
+        if (active) store_out(out + k, fx_scale<UNIT>(x, k == 0 ? se : sm));
     };
     if constexpr (NT <= 32) {
         const int src = (NT - j) & (NT - 1);
@@ -221,29 +259,31 @@ __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, uns
         });
     }
     if (active && j == 0) {
-        double x = fx_to(v[0].x - v[0].y, e);
-        if (!unit) x *= se;
-        out[M] = cmake<double2>(x, 0.0);
+        out[M] = fx_scale<UNIT>(cmake<double2>(fx_to(v[0].x - v[0].y, e), 0.0), se);
     }
 }
 
 // Output scale s of a C2R line as an exponent where it is a power of two (the
-// factor left over is then 1).
-__device__ __forceinline__ double fx_split_scale(double s, int &e)
+// factor left over is then 1; UNIT kernels run only then, see fx_unit_scale).
+inline bool fx_unit_scale(double s)
 {
     const uint64_t u = fx_bits(s);
-    const int ex = (int)(u >> 52 & 0x7ff);
-    if ((u & 0xfffffffffffffULL) == 0 && ex > 1023 - 100 && ex < 1023 + 100) {
-        e += ex - 1023;
+    return (u & 0xfffffffffffffULL) == 0 && u >> 52 > 1023 - 100 && u >> 52 < 1023 + 100;
+}
+template <bool UNIT> __device__ __forceinline__ double fx_split_scale(double s, int &e)
+{
+    if constexpr (UNIT) {
+        e += (int)(fx_bits(s) >> 52) - 1023;
         return 1.0;
+    } else {
+        return s;
     }
-    return s;
 }
 
 // zc2r_lines in fixed point.  The pre-process at most quadruples a thread's L1
 // norm (its own entries and their mirror images, twice each), so the entries
 // come in at 2^-2 of the usual scale; its rotation by r / 4 acts on 4 d.
-template <int M, int E, int LPB>
+template <int M, int E, int LPB, bool UNIT>
 __device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, unsigned char *smem,
                                               const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
 {
@@ -330,21 +370,15 @@ __device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, uns
     line_fft<fx64, M, E>(v, j, tw, ex);
 
     int e = g - 1023 - (kFxBits - 2) + fx_line_shift<M, E>();
-    const double f = fx_split_scale(a.scale_mid, e);
+    const double f = fx_split_scale<UNIT>(a.scale_mid, e);
     double2 *out = (double2 *)((double *)a.real_out + l * a.real_pitch);
-    if (active) {
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            double2 o = fx_out(cconj(v[i]), e);
-            if (f != 1.0) o = cscale(o, f);
-            store_out(out + j + i * NT, o);
-        }
-    }
+    if (active)
+        fx_out_all<E>(v, e, [&](int i, double2 o) { store_out(out + j + i * NT, fx_scale<UNIT>(cconj(o), f)); });
 }
 
 // zr2c_pairs in fixed point; the two lines share a scale, as they share the
 // FP64 form's rounding errors.
-template <int M, int E, int LPB>
+template <int M, int E, int LPB, bool UNIT>
 __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, unsigned char *smem,
                                               const fxtw *__restrict__ tw)
 {
@@ -387,21 +421,17 @@ __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, uns
     double2 *out1 = out0 + (M + 1);
     const int e = g - 1023 - kFxBits + fx_line_shift<N, E>() - 1;
     const double se = a.scale_edge, sm = a.scale_mid;
-    const bool unit = se == 1.0 && sm == 1.0;
     static_for<0, M / NT + 1>([&](auto II) {
         constexpr int i = decltype(II)::value;
         if (i < M / NT || j == 0) {
             const int k = j + i * NT;
             const fxc z = v[i];
             const fxc zm = (k == 0 || k == M) ? z : ex.get(pad_row<P, LREV>(N - j, -i * NT));  // Z[N - k]
-            double2 x0 = fx_out(fx_make(z.x + zm.x, z.y - zm.y), e), x1 = fx_out(fx_make(z.y + zm.y, zm.x - z.x), e);
-            if (!unit) {
-                const double f = (k == 0 || k == M) ? se : sm;
-                x0 = cscale(x0, f);
-                x1 = cscale(x1, f);
-            }
-            if (act0) store_out(out0 + k, x0);
-            if (act1) store_out(out1 + k, x1);
+            const double2 x0 = fx_out(fx_make(z.x + zm.x, z.y - zm.y), e),
+                          x1 = fx_out(fx_make(z.y + zm.y, zm.x - z.x), e);
+            const double f = (k == 0 || k == M) ? se : sm;
+            if (act0) store_out(out0 + k, fx_scale<UNIT>(x0, f));
+            if (act1) store_out(out1 + k, fx_scale<UNIT>(x1, f));
         }
     });
 }
@@ -409,7 +439,7 @@ __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, uns
 // zc2r_pairs in fixed point.  Thread j converts the entries k = j + i NT < M of
 // both lines once; they give Z[k] = x0 + i x1, its own, and Z[N - k] =
 // conj x0 + i conj x1, which another thread of the pair owns.
-template <int M, int E, int LPB>
+template <int M, int E, int LPB, bool UNIT>
 __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, unsigned char *smem,
                                               const fxtw *__restrict__ tw)
 {
@@ -478,36 +508,34 @@ __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, uns
     line_fft<fx64, N, E>(v, j, tw, ex);
 
     int e = g - 1023 - (kFxBits - 1) + fx_line_shift<N, E>();
-    const double f = fx_split_scale(a.scale_mid, e);
+    const double f = fx_split_scale<UNIT>(a.scale_mid, e);
     double *out0 = (double *)a.real_out + la * a.real_pitch;
     double *out1 = (double *)a.real_out + lb * a.real_pitch;
-#pragma unroll
-    for (int i = 0; i < E; ++i) {
-        double2 z = fx_out(cswap(v[i]), e);  // x0 + i x1 at n = j + i NT
-        if (f != 1.0) z = cscale(z, f);
-        if (act0) store_out(out0 + j + i * NT, z.x);
-        if (act1) store_out(out1 + j + i * NT, z.y);
-    }
+    fx_out_all<E>(v, e, [&](int i, double2 o) {  // x1 + i x0 at n = j + i NT
+        const double2 z = fx_scale<UNIT>(o, f);
+        if (act0) store_out(out0 + j + i * NT, z.y);
+        if (act1) store_out(out1 + j + i * NT, z.x);
+    });
 }
 
 // A group of LPB lines, by the form that serves the length.
-template <typename R, int M, int E, int LPB, bool PF>
+template <typename R, int M, int E, int LPB, bool PF, bool UNIT>
 __device__ __forceinline__ void zr2c_group(const ZArgs &a, int64_t line0, unsigned char *smem,
                                            const typename twvec<R>::T *__restrict__ tw,
                                            const typename twvec<R>::T *__restrict__ rot)
 {
     if constexpr (!z_fixed<R, M>()) zr2c_lines<R, M, E, LPB, PF>(a, line0, smem, tw, rot);
-    else if constexpr (z_paired<R, M>()) zr2c_fx_pairs<M, E, LPB>(a, line0, smem, tw);
-    else zr2c_fx_lines<M, E, LPB>(a, line0, smem, tw, rot);
+    else if constexpr (z_paired<R, M>()) zr2c_fx_pairs<M, E, LPB, UNIT>(a, line0, smem, tw);
+    else zr2c_fx_lines<M, E, LPB, UNIT>(a, line0, smem, tw, rot);
 }
-template <typename R, int M, int E, int LPB, bool PF>
+template <typename R, int M, int E, int LPB, bool PF, bool UNIT>
 __device__ __forceinline__ void zc2r_group(const ZArgs &a, int64_t line0, unsigned char *smem,
                                            const typename twvec<R>::T *__restrict__ tw,
                                            const typename twvec<R>::T *__restrict__ rot)
 {
     if constexpr (!z_fixed<R, M>()) zc2r_lines<R, M, E, LPB, false, PF>(a, line0, smem, tw, rot);
-    else if constexpr (z_paired<R, M>()) zc2r_fx_pairs<M, E, LPB>(a, line0, smem, tw);
-    else zc2r_fx_lines<M, E, LPB>(a, line0, smem, tw, rot);
+    else if constexpr (z_paired<R, M>()) zc2r_fx_pairs<M, E, LPB, UNIT>(a, line0, smem, tw);
+    else zc2r_fx_lines<M, E, LPB, UNIT>(a, line0, smem, tw, rot);
 }
 
 // One group of LPB lines per block; with LOOP, a grid of a.max_blocks blocks
@@ -522,12 +550,15 @@ __device__ __forceinline__ void zc2r_group(const ZArgs &a, int64_t line0, unsign
 // slower, and for the C2R kernel, or powers of two, it raises registers.
 template <typename R, int M, int E> __host__ __device__ constexpr int zr2c_minb()
 {
-    return sizeof(R) == 4 ? (E == 24 && M >= 384 ? 1 : 0) : (z_fixed<R, M>() ? 2 : 0);
+    return sizeof(R) == 4 && E == 24 && M >= 384 ? 1 : 0;
 }
-template <typename R, int M> __host__ __device__ constexpr int zc2r_minb() { return z_fixed<R, M>() ? 2 : 0; }
+template <typename R, int M, int E, int LPB> __host__ __device__ constexpr int fx_z_minb()
+{
+    return z_fixed<R, M>() ? fx_min_blocks(E, LPB * (M / E)) : 0;
+}
 
-template <typename R, int M, int E, int LPB, bool LOOP>
-__global__ void __launch_bounds__(LPB *(M / E), zr2c_minb<R, M, E>())
+template <typename R, int M, int E, int LPB, bool LOOP, bool UNIT>
+__global__ void __launch_bounds__(LPB *(M / E), sizeof(R) == 8 ? fx_z_minb<R, M, E, LPB>() : zr2c_minb<R, M, E>())
 zpass_r2c_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
                  const typename twvec<R>::T *__restrict__ rot)
 {
@@ -535,15 +566,15 @@ zpass_r2c_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__
     if constexpr (LOOP) {
         for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
             if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
-            zr2c_group<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
+            zr2c_group<R, M, E, LPB, false, false>(a, blk * LPB, smem_raw, tw, rot);
         }
     } else {
-        zr2c_group<R, M, E, LPB, z_l2pf<R, M, false>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+        zr2c_group<R, M, E, LPB, z_l2pf<R, M, false>(), UNIT>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
     }
 }
 
-template <typename R, int M, int E, int LPB, bool LOOP>
-__global__ void __launch_bounds__(LPB *(M / E), zc2r_minb<R, M>())
+template <typename R, int M, int E, int LPB, bool LOOP, bool UNIT>
+__global__ void __launch_bounds__(LPB *(M / E), fx_z_minb<R, M, E, LPB>())
 zpass_c2r_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
                  const typename twvec<R>::T *__restrict__ rot)
 {
@@ -551,10 +582,10 @@ zpass_c2r_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__
     if constexpr (LOOP) {
         for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
             if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
-            zc2r_group<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
+            zc2r_group<R, M, E, LPB, false, false>(a, blk * LPB, smem_raw, tw, rot);
         }
     } else {
-        zc2r_group<R, M, E, LPB, z_l2pf<R, M, true>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+        zc2r_group<R, M, E, LPB, z_l2pf<R, M, true>(), UNIT>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
     }
 }
 

@@ -250,8 +250,8 @@ constexpr int kFxMinCode = 128, kFxMaxCode = 1900, kFxZeroCode = 1023;
 FX_HD float fx_mag(int32_t top, int32_t expo)  // |v| / 2^(expo's exponent), at least 2^-100
 {
     const int32_t fl = expo - (100 << 20);
-    const int32_t t = top > fl ? top : fl;
-    return fx_float((uint32_t)(t - expo + (127 << 20)) << 3);
+    const uint32_t t = (uint32_t)(top > fl ? top : fl);
+    return fx_float(t * 8u + ((127u << 20) - (uint32_t)expo) * 8u);
 }
 FX_HD int fx_code(int32_t top_max, float sum)
 {
@@ -269,30 +269,58 @@ FX_HD int64_t fx_from(double v, int g, int bits)
     const uint64_t u = fx_bits(v);
     const uint32_t hi = (uint32_t)(u >> 32);
     const uint64_t m = (u << 11) | 0x8000000000000000ULL;
-    const uint32_t sh = (uint32_t)(g + (63 - bits)) - (hi >> 20 & 0x7ffu);
+    const uint32_t sh = (uint32_t)(g + (63 - bits)) - ((hi & 0x7fffffffu) >> 20);
 #ifdef __CUDA_ARCH__
-    uint64_t a;
-    asm("shr.u64 %0, %1, %2;" : "=l"(a) : "l"(m), "r"(sh));  // 0 from 64 on
+    int64_t a;
+    asm("{\n .reg .pred p;\n shr.u64 %0, %1, %2;\n"  // 0 from 64 on
+        " setp.lt.s32 p, %3, 0;\n @p neg.s64 %0, %0;\n}\n"
+        : "=&l"(a)
+        : "l"(m), "r"(sh), "r"((int32_t)hi));
+    return a;
 #else
     const uint64_t a = sh > 63 ? 0 : m >> sh;
-#endif
     return (int32_t)hi < 0 ? -(int64_t)a : (int64_t)a;
+#endif
 }
 
-// X 2^e, rounded to nearest, for |X| < 2^62 and e in [-1000, 900].  Two ways to
-// the same value (up to ties): fx_to on the integer pipe, fx_to_fp with two
-// FP64 additions.
-FX_HD double fx_to(int64_t X, int e)
+// Position of the leading bit of h that differs from its sign, -1 without one.
+FX_HD int32_t fx_lead(int32_t h)
 {
-    const uint64_t a = X < 0 ? (uint64_t)(-X) : (uint64_t)X;
-    const int lz = fx_clz(a);
-    // 53 bits (or 2^53), leading bit set; ties go up, also for negative X, so that they leave no bias
-    const uint64_t r = ((a << (lz - 1)) + (X < 0 ? 511 : 512)) >> 10;
-    uint32_t hi = (uint32_t)(r >> 32) + ((uint32_t)(e + 1085 - lz) << 20);
-    hi |= (uint32_t)((uint64_t)X >> 32) & 0x80000000u;
-    return a == 0 ? 0.0 : fx_double((uint64_t)hi << 32 | (uint32_t)r);
+#ifdef __CUDA_ARCH__
+    int32_t p;
+    asm("bfind.s32 %0, %1;" : "=r"(p) : "r"(h));
+    return p;
+#else
+    const uint32_t a = (uint32_t)(h ^ (h >> 31));
+    return a ? 31 - __builtin_clz(a) : -1;
+#endif
 }
-FX_HD double fx_to_fp(int64_t X, int e)
+FX_HD uint32_t fx_shl_hi(uint32_t lo, uint32_t hi, uint32_t n)  // high word of hi:lo << n, n < 32
+{
+#ifdef __CUDA_ARCH__
+    return __funnelshift_l(lo, hi, n);
+#else
+    return n ? hi << n | lo >> (32 - n) : hi;
+#endif
+}
+
+// X 2^e, rounded to nearest (ties towards +infinity, so that they leave no
+// bias), for |X| < 2^62 and e in [-1000, 900], on the integer pipe.  Serves
+// |X| >= 2^32, else clears the sign bit of `big` and returns anything.
+FX_HD double fx_to_big(int64_t X, int e, int32_t &big)
+{
+    const uint32_t hi = (uint32_t)((uint64_t)X >> 32), lo = (uint32_t)(uint64_t)X;
+    const uint32_t s = (uint32_t)((int32_t)hi >> 31);
+    const int32_t p = fx_lead((int32_t)hi);
+    big &= ~p;
+    const uint32_t n = (uint32_t)(30 - p) & 31;
+    // |X| 2^n with its leading bit at 62 (one less in the last place if X < 0)
+    const uint64_t v = ((uint64_t)(fx_shl_hi(lo, hi, n) ^ s) << 32 | ((lo << n) ^ s)) + 512;
+    const uint32_t r = (uint32_t)(v >> 42) + ((uint32_t)p << 20);
+    return fx_double((uint64_t)(r + (((uint32_t)(e + 1054) << 20) | (s & 0x80000000u))) << 32 | (uint32_t)(v >> 10));
+}
+// The same for any |X| < 2^62, with two FP64 additions (ties to even).
+FX_HD double fx_to(int64_t X, int e)
 {
     const uint32_t s = (uint32_t)e << 20;
     const double dh = fx_double((uint64_t)(0x45300000u + s) << 32 | ((uint32_t)((uint64_t)X >> 32) ^ 0x80000000u));

@@ -78,40 +78,61 @@ __host__ __device__ constexpr bool pair_axis(int axis) { return axis >= 0 && ((F
 constexpr int kPairW = 16;  // columns of a CTA-pair tile (128-byte float rows)
 
 // Elements per thread of a column pass: 32 in the pipelined kernel, else the
-// default plan of the length; double columns of 512 points take 8 (radix 8 x 8
-// x 8, fewer twiddle products than 16 x 16 x 2, on 4-column tiles).
+// default plan of the length; double columns of up to 512 = 2^k points take 8:
+// 64 registers a thread, so 1024 threads an SM hide the latencies of the
+// integer pipe that 512 threads of 16 elements leave open, and a small grid
+// finishes sooner.  Measured on GB300: 512^3 y-pass 0.78 -> 0.64 ms, 64^3 pair
+// 71 -> 55 us; at 1024 points (a third exchange, 512-thread blocks) 6.1 -> 6.7 ms.
 template <typename R, int L> __host__ __device__ constexpr int col_E()
 {
-    return col_pipe<R, L>() ? 32 : ((sizeof(R) == 8 && L == 512) ? 8 : line_E(L));
+    return col_pipe<R, L>() ? 32 : ((sizeof(R) == 8 && is_pow2(L) && L >= 8 && L <= 512) ? 8 : line_E(L));
+}
+
+// Columns per tile of a fixed-point column pass along axis AX: 256 threads a
+// block (128 for 3 * 2^k <= 384, whose 24-element threads then keep 168
+// registers instead of spilling: 192-point columns 0.064 -> 0.053 ms at
+// 192 x 128 x 384), at most a warp's worth.  The x-pass of 512 points takes 8
+// columns and 512 threads: its rows lie N1 (N2/2+1) entries apart, where a copy
+// in 64-byte row segments reaches 3.1-3.7 TB/s and one in 128-byte segments
+// 5.7-6 (512^3: 0.70 -> 0.68 ms, 512 x 512 x 2048: 3.03 -> 2.67; the y-pass
+// loses, 0.64 -> 0.72).
+template <typename R, int L, int AX> __host__ __device__ constexpr int col_fx_W()
+{
+    constexpr int nt = L / col_E<R, L>();
+    constexpr int t = AX == 0 && L == 512 ? 512 : line_E(L) == 24 && L <= 384 ? 128 : 256;
+    return t / nt < 32 ? t / nt : 32;
 }
 
 // Columns per tile: one 128-byte segment per row (16 float2 or 8 double2),
 // halved while the block would exceed its thread cap or, for the one-tile
 // kernel, the tile 200 KB of shared memory.
-template <typename R, int L> __host__ __device__ constexpr int col_W()
+template <typename R, int L, int AX = 1> __host__ __device__ constexpr int col_W()
 {
     int w = 128 / (int)sizeof(typename cvec<R>::T);
     if (col_pipe<R, L>()) {
         while (w > 1 && w * (L / 32) > 512) w /= 2;
         return w;
     }
-    if (col_fixed<R, L>() && L / col_E<R, L>() < 8) w = 32;  // at least a warp per block
+    if (col_fixed<R, L>()) return col_fx_W<R, L, AX>();
     while (w > 1 && (w * (L / col_E<R, L>()) > col_max_threads<R, L>() ||
                      (size_t)L * w * sizeof(typename cvec<R>::T) > 200 * 1024))
         w /= 2;
     return w;
 }
 
-// Lines per block of a z pass: about 256 threads, and at least one warp.
+// Lines per block of a z pass: about 256 threads (128 for double lines of 24
+// elements a thread, which then keep 168 registers; measured at 768^3 3.9 -> 3.3
+// ms a pass), and at least one warp.
 template <typename R, int M> __host__ __device__ constexpr int z_LPB()
 {
-    return M / z_E<R, M>() >= FFT3D_Z_THREADS ? 1 : FFT3D_Z_THREADS / (M / z_E<R, M>());
+    const int t = sizeof(R) == 8 && z_E<R, M>() == 24 ? 128 : FFT3D_Z_THREADS;
+    return M / z_E<R, M>() >= t ? 1 : t / (M / z_E<R, M>());
 }
 
 template <typename R, int L> inline void col_geom_t(PassGeom *g, int axis)
 {
-    constexpr int W = col_W<R, L>();
     constexpr int E = col_E<R, L>();
+    const int W = axis == 0 ? col_W<R, L, 0>() : col_W<R, L, 1>();
     g->threads = W * (L / E);
     g->per_block = W;
     g->E = E;
@@ -131,9 +152,9 @@ template <typename R, int L> inline void col_geom_t(PassGeom *g, int axis)
         }
     }
     if (col_pipe<R, L>())
-        g->smem = pipe_smem_bytes<R, L, E, W>();
+        g->smem = pipe_smem_bytes<R, L, E, col_W<R, L>()>();
     else if (xstage)
-        g->smem = xstage_smem_bytes<R, L, E, W>();
+        g->smem = xstage_smem_bytes<R, L, E, col_W<R, L>()>();
     else
         g->smem = (size_t)L * W * sizeof(C) + (col_fixed<R, L>() ? W * sizeof(int) : 0);  // and the scale codes
 }
@@ -152,11 +173,11 @@ template <typename R, int M> inline void z_geom_t(PassGeom *g)
               sizeof(typename cvec<R>::T);
 }
 
-// The kernel that runs one column tile per block.
-template <typename R, int L, bool INV> inline auto col_one_tile_kernel()
+// The kernel that runs one column tile per block along axis AX.
+template <typename R, int L, int AX, bool INV> inline auto col_one_tile_kernel()
 {
-    if constexpr (col_fixed<R, L>()) return colpass_fx_kernel<L, col_E<R, L>(), col_W<R, L>(), INV>;
-    else return colpass_kernel<R, L, col_E<R, L>(), col_W<R, L>(), INV>;
+    if constexpr (col_fixed<R, L>()) return colpass_fx_kernel<L, col_E<R, L>(), col_W<R, L, AX>(), INV>;
+    else return colpass_kernel<R, L, col_E<R, L>(), col_W<R, L, AX>(), INV>;
 }
 
 template <typename R, int L> inline cudaError_t col_prepare_t()
@@ -198,23 +219,38 @@ template <typename R, int L> inline cudaError_t col_prepare_t()
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, xs);
             if (e != cudaSuccess) return e;
         }
-        e = cudaFuncSetAttribute(col_one_tile_kernel<R, L, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)g.smem);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(col_one_tile_kernel<R, L, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)g.smem);
+        const void *const ks[4] = {(const void *)col_one_tile_kernel<R, L, 0, false>(),
+                                   (const void *)col_one_tile_kernel<R, L, 0, true>(),
+                                   (const void *)col_one_tile_kernel<R, L, 1, false>(),
+                                   (const void *)col_one_tile_kernel<R, L, 1, true>()};
+        PassGeom g0;
+        col_geom_t<R, L>(&g0, 0);
+        const size_t one_tile = g0.persistent || g0.smem < g.smem ? g.smem : g0.smem;
+        for (const void *k : ks) {
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one_tile);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
     }
+}
+
+// z kernels of a length: [LOOP, UNIT]; UNIT only for double lines without LOOP.
+template <typename R, int M, bool C2R, bool LOOP, bool UNIT> inline auto z_kernel()
+{
+    constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
+    constexpr bool U = UNIT && z_fixed<R, M>();
+    if constexpr (C2R) return zpass_c2r_kernel<R, M, E, LPB, LOOP, U>;
+    else return zpass_r2c_kernel<R, M, E, LPB, LOOP, U>;
 }
 
 template <typename R, int M> inline cudaError_t z_prepare_t()
 {
     PassGeom g;
     z_geom_t<R, M>(&g);
-    constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
-    const void *const ks[4] = {(const void *)zpass_r2c_kernel<R, M, E, LPB, false>,
-                               (const void *)zpass_r2c_kernel<R, M, E, LPB, true>,
-                               (const void *)zpass_c2r_kernel<R, M, E, LPB, false>,
-                               (const void *)zpass_c2r_kernel<R, M, E, LPB, true>};
+    const void *const ks[6] = {
+        (const void *)z_kernel<R, M, false, false, false>(), (const void *)z_kernel<R, M, false, true, false>(),
+        (const void *)z_kernel<R, M, true, false, false>(),  (const void *)z_kernel<R, M, true, true, false>(),
+        (const void *)z_kernel<R, M, false, false, true>(),  (const void *)z_kernel<R, M, true, false, true>()};
     for (const void *k : ks) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
         if (e != cudaSuccess) return e;
@@ -364,7 +400,8 @@ inline cudaError_t col_launch_t(const ColArgs &a, int64_t tiles, const void *tw,
                 return cudaGetLastError();
             }
         }
-        auto k = a.inverse ? col_one_tile_kernel<R, L, true>() : col_one_tile_kernel<R, L, false>();
+        auto k = a.axis == 0 ? (a.inverse ? col_one_tile_kernel<R, L, 0, true>() : col_one_tile_kernel<R, L, 0, false>())
+                             : (a.inverse ? col_one_tile_kernel<R, L, 1, true>() : col_one_tile_kernel<R, L, 1, false>());
         ColArgs b = a;
         b.pf_stride = col_l2_prefetch<R, L>(a.axis) ? persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) : 0;
         k<<<(unsigned)tiles, g.threads, g.smem, st>>>(b, (TW)tw);
@@ -377,15 +414,15 @@ inline cudaError_t zr2c_launch_t(const ZArgs &a, const void *tw, const void *rot
 {
     PassGeom g;
     z_geom_t<R, M>(&g);
-    constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
     const int64_t blocks = (a.nlines + g.per_block - 1) / g.per_block;
     typedef const typename twvec<R>::T *TW;
     if (a.max_blocks > 0 && blocks > a.max_blocks)
-        zpass_r2c_kernel<R, M, E, LPB, true><<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
+        z_kernel<R, M, false, true, false>()<<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
     else {
-        auto k = zpass_r2c_kernel<R, M, E, LPB, false>;
+        const bool unit = a.scale_edge == 1.0 && a.scale_mid == 1.0;
+        auto k = unit ? z_kernel<R, M, false, false, true>() : z_kernel<R, M, false, false, false>();
         ZArgs b = a;
-        b.pf_lines = z_l2pf<R, M, false>() ? (int64_t)persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) * LPB : 0;
+        b.pf_lines = z_l2pf<R, M, false>() ? (int64_t)persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) * g.per_block : 0;
         k<<<(unsigned)blocks, g.threads, g.smem, st>>>(b, (TW)tw, (TW)rot);
     }
     return cudaGetLastError();
@@ -396,15 +433,15 @@ inline cudaError_t zc2r_launch_t(const ZArgs &a, const void *tw, const void *rot
 {
     PassGeom g;
     z_geom_t<R, M>(&g);
-    constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
     const int64_t blocks = (a.nlines + g.per_block - 1) / g.per_block;
     typedef const typename twvec<R>::T *TW;
     if (a.max_blocks > 0 && blocks > a.max_blocks)
-        zpass_c2r_kernel<R, M, E, LPB, true><<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
+        z_kernel<R, M, true, true, false>()<<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
     else {
-        auto k = zpass_c2r_kernel<R, M, E, LPB, false>;
+        const bool unit = fx_unit_scale(a.scale_mid);
+        auto k = unit ? z_kernel<R, M, true, false, true>() : z_kernel<R, M, true, false, false>();
         ZArgs b = a;
-        b.pf_lines = z_l2pf<R, M, true>() ? (int64_t)persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) * LPB : 0;
+        b.pf_lines = z_l2pf<R, M, true>() ? (int64_t)persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) * g.per_block : 0;
         k<<<(unsigned)blocks, g.threads, g.smem, st>>>(b, (TW)tw, (TW)rot);
     }
     return cudaGetLastError();

@@ -1011,9 +1011,15 @@ struct ZArgs {
 // 45% slower.
 // Double lines of N2 = 1024 points (M = 512) run two lines per complex
 // transform of N2 points (z_paired; 16 elements per thread, radix 16 x 16 x 4):
-// no Hermitian rotation, one twiddle product per element fewer.
+// no Hermitian rotation, one twiddle product per element fewer.  Double lines
+// of up to 128 = 2^k points take 8 elements per thread (64 registers): small
+// grids finish sooner (64^3: 14 -> 10 us a pass), and it makes no difference at
+// 256 points and loses 5% at 1024.
 template <typename R, int M> __host__ __device__ constexpr bool z_paired() { return sizeof(R) == 8 && M == 512; }
-template <typename R, int M> __host__ __device__ constexpr int z_E() { return z_paired<R, M>() ? 16 : line_E(M); }
+template <typename R, int M> __host__ __device__ constexpr int z_E()
+{
+    return z_paired<R, M>() ? 16 : sizeof(R) == 8 && is_pow2(M) && M >= 8 && M <= 128 ? 8 : line_E(M);
+}
 
 // Per-line shared-memory exchange with one padding slot every 2^P elements:
 // P = 4 makes the stride-16 writes of a radix-16 first stage conflict-free;
