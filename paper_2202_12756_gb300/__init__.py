@@ -101,6 +101,9 @@ def _declare(lib):
 def load_library(path=LIB_PATH):
     """Load libfft3d.so (built by ``__graft_entry__.build()`` or ``_build.py``)."""
     global _lib
+    lib = _lib
+    if lib is not None and path == LIB_PATH:
+        return lib
     with _lib_lock:
         if _lib is None or path != LIB_PATH:
             if not os.path.exists(path):
@@ -254,9 +257,20 @@ def fft3d_measure_fp64_peak():
 
 
 # ------------------------------------------------------------ torch layer
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+def _raw_stream(index):
+    """cudaStream_t of torch's current stream on device `index`, without a Stream object."""
+    return _torch()._C._cuda_getCurrentRawStream(index)
 
 
 def _dtype_code(real_dtype):
@@ -293,6 +307,10 @@ class Plan:
         self.device = torch.device(device if device is not None else "cuda", )
         if self.device.index is None:
             self.device = torch.device("cuda", torch.cuda.current_device())
+        n0, n1, n2 = self.shape
+        self._real = self.lead + self.shape
+        self._half = self.lead + (n0, n1, n2 // 2 + 1)
+        self._padded = self.lead + (n0, n1, 2 * (n2 // 2 + 1))
         with torch.cuda.device(self.device):
             self.handle = fft3d_plan_create_batched(self.batch, *self.shape, _dtype_code(dtype))
 
@@ -307,20 +325,20 @@ class Plan:
 
     @property
     def half_shape(self):
-        n0, n1, n2 = self.shape
-        return self.lead + (n0, n1, n2 // 2 + 1)
+        return self._half
 
     @property
     def real_shape(self):
-        return self.lead + self.shape
-
-    def _stream(self):
-        return _torch().cuda.current_stream(self.device).cuda_stream
+        return self._real
 
     def _run(self, fn, src, dst):
-        torch = _torch()
-        with torch.cuda.device(self.device):
-            fn(self.handle, src.data_ptr(), dst.data_ptr(), self._stream())
+        cuda = _torch().cuda
+        index = self.device.index
+        if cuda.current_device() == index:
+            fn(self.handle, src.data_ptr(), dst.data_ptr(), _raw_stream(index))
+            return
+        with cuda.device(self.device):
+            fn(self.handle, src.data_ptr(), dst.data_ptr(), _raw_stream(index))
 
     def empty_real(self):
         return _torch().empty(self.real_shape, dtype=self.real_dtype, device=self.device)
@@ -330,19 +348,16 @@ class Plan:
 
     def empty_padded(self):
         """Real buffer with rows padded to 2 (N2/2 + 1): the in-place layout."""
-        n0, n1, n2 = self.shape
-        return _torch().empty(self.lead + (n0, n1, 2 * (n2 // 2 + 1)), dtype=self.real_dtype,
-                              device=self.device)
+        return _torch().empty(self._padded, dtype=self.real_dtype, device=self.device)
 
     def _check_real(self, t, padded=False, host_ok=False):
-        n0, n1, n2 = self.shape
-        want = self.lead + ((n0, n1, 2 * (n2 // 2 + 1)) if padded else self.shape)
+        want = self._padded if padded else self._real
         where_ok = t.device == self.device or (host_ok and t.device.type == "cpu" and t.is_pinned())
-        if t.dtype != self.real_dtype or tuple(t.shape) != want or not t.is_contiguous() or not where_ok:
+        if t.dtype != self.real_dtype or t.shape != want or not t.is_contiguous() or not where_ok:
             raise FFT3DError(FFT3D_ERR_ARG, "real tensor", f"need contiguous {want} {self.real_dtype} on {self.device}")
 
     def _check_cplx(self, t):
-        if (t.dtype != self.complex_dtype or tuple(t.shape) != self.half_shape or not t.is_contiguous()
+        if (t.dtype != self.complex_dtype or t.shape != self._half or not t.is_contiguous()
                 or t.device != self.device):
             raise FFT3DError(FFT3D_ERR_ARG, "complex tensor",
                              f"need contiguous {self.half_shape} {self.complex_dtype} on {self.device}")
@@ -350,15 +365,19 @@ class Plan:
     # out-of-place; x may also be a pinned host tensor (read once, by the first pass)
     def r2c(self, x, out=None):
         self._check_real(x, host_ok=True)
-        out = self.empty_complex() if out is None else out
-        self._check_cplx(out)
+        if out is None:
+            out = self.empty_complex()
+        else:
+            self._check_cplx(out)
         self._run(fft3d_exec_r2c, x, out)
         return out
 
     def c2r(self, X, out=None):
         self._check_cplx(X)
-        out = self.empty_real() if out is None else out
-        self._check_real(out)
+        if out is None:
+            out = self.empty_real()
+        else:
+            self._check_real(out)
         self._run(fft3d_exec_c2r, X, out)
         return out
 
@@ -373,15 +392,19 @@ class Plan:
 
     def r2c_adjoint(self, G, out=None):
         self._check_cplx(G)
-        out = self.empty_real() if out is None else out
-        self._check_real(out)
+        if out is None:
+            out = self.empty_real()
+        else:
+            self._check_real(out)
         self._run(fft3d_exec_r2c_adjoint, G, out)
         return out
 
     def c2r_adjoint(self, g, out=None):
         self._check_real(g)
-        out = self.empty_complex() if out is None else out
-        self._check_cplx(out)
+        if out is None:
+            out = self.empty_complex()
+        else:
+            self._check_cplx(out)
         self._run(fft3d_exec_c2r_adjoint, g, out)
         return out
 
@@ -433,11 +456,15 @@ def get_plan(shape, dtype, device, batch=1):
     plane and tile counter are shared by its calls), so each stream gets a
     plan of its own."""
     torch = _torch()
-    device = torch.device(device)
+    if not isinstance(device, torch.device):
+        device = torch.device(device)
     if device.index is None:
         device = torch.device("cuda", torch.cuda.current_device())
-    stream = torch.cuda.current_stream(device).cuda_stream
-    key = (tuple(int(s) for s in shape), dtype, device.index, int(batch), stream)
+    stream = _raw_stream(device.index) if device.type == "cuda" else torch.cuda.current_stream(device).cuda_stream
+    key = (tuple(map(int, shape)), dtype, device.index, int(batch), stream)
+    p = _plans.get(key)
+    if p is not None:
+        return p
     with _plans_lock:
         p = _plans.get(key)
         if p is None:
@@ -448,7 +475,7 @@ def get_plan(shape, dtype, device, batch=1):
 
 def _split_batch(shape):
     """(batch, field shape) of a 3D shape or a 4D [B, N0, N1, N2] shape."""
-    shape = tuple(int(s) for s in shape)
+    shape = tuple(map(int, shape))
     if len(shape) == 4:
         return shape[0], shape[1:]
     if len(shape) == 3:
