@@ -106,6 +106,7 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
     constexpr int NT = L / E;
     static_assert(W <= 32 && W * NT % 32 == 0, "a warp holds all columns of the tile");
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pass_begin();
     int *code = (int *)(smem_raw + (size_t)L * W * sizeof(fxc));
     const int c = threadIdx.x % W;
     const int j = threadIdx.x / W;
@@ -149,6 +150,7 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
     }
     ColEx<fxc, W> ex{(fxc *)smem_raw, c};
     line_fft<fx64, L, E>(v, j, tw, ex);
+    pass_release();
     const int e = g - 1023 - kFxBits + fx_line_shift<L, E>();
     if (valid) {
         double2 *dj = dp + (int64_t)j * ds;
@@ -227,6 +229,7 @@ __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, uns
         for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
     }
     line_fft<fx64, M, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     const int e = g - 1023 - kFxBits + fx_line_shift<M, E>();
     double2 *out = (double2 *)a.cplx.main + (active ? line : 0) * (M + 1);
@@ -368,6 +371,7 @@ __device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, uns
         ex.sync();
     }
     line_fft<fx64, M, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     int e = g - 1023 - (kFxBits - 2) + fx_line_shift<M, E>();
     const double f = fx_split_scale<UNIT>(a.scale_mid, e);
@@ -411,6 +415,7 @@ __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, uns
         for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
     }
     line_fft<fx64, N, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     constexpr bool LR = pad_linear_reads<P>(NT);
     constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
@@ -506,6 +511,7 @@ __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, uns
         ex.sync();
     }
     line_fft<fx64, N, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     int e = g - 1023 - (kFxBits - 1) + fx_line_shift<N, E>();
     const double f = fx_split_scale<UNIT>(a.scale_mid, e);
@@ -563,6 +569,7 @@ zpass_r2c_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__
                  const typename twvec<R>::T *__restrict__ rot)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pass_begin();
     if constexpr (LOOP) {
         for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
             if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
@@ -579,6 +586,7 @@ zpass_c2r_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__
                  const typename twvec<R>::T *__restrict__ rot)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pass_begin();
     if constexpr (LOOP) {
         for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
             if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group

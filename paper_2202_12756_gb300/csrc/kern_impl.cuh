@@ -258,6 +258,28 @@ template <typename R, int M> inline cudaError_t z_prepare_t()
     return cudaSuccess;
 }
 
+// Launches a pass kernel so that its blocks are set up while the kernel before
+// it on the stream drains (programmatic dependent launch; see pass_begin).
+template <class... P, class... A>
+inline cudaError_t launch_pass(void (*k)(P...), int64_t grid, int threads, size_t smem, cudaStream_t st, const A &...args)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    memset(&attr, 0, sizeof(attr));
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // reported here, not to the caller's next check
+    return e;
+}
+
 // Resident blocks of a persistent kernel on the current device, cached per
 // (kernel, device), capped at the blocks that get work: `items` work items
 // taken `per_block_items` at a time.
@@ -367,8 +389,7 @@ inline cudaError_t col_launch_t(const ColArgs &a, int64_t tiles, const void *tw,
             else memset(&map, 0, sizeof(map));
             if (tmap2) map2 = *tmap2;
             else memset(&map2, 0, sizeof(map2));
-            k<<<grid, g.threads, g.smem, st>>>(a, (TW)tw, tiles, map, map2);
-            return cudaGetLastError();
+            return launch_pass(k, grid, g.threads, g.smem, st, a, (TW)tw, tiles, map, map2);
         }
     }
     if constexpr (col_pipe<R, L>()) {
@@ -383,7 +404,7 @@ inline cudaError_t col_launch_t(const ColArgs &a, int64_t tiles, const void *tw,
         else memset(&map, 0, sizeof(map));
         if (tmap2) map2 = *tmap2;
         else memset(&map2, 0, sizeof(map2));
-        k<<<grid, g.threads, g.smem, st>>>(a, (TW)tw, tiles, map, map2);
+        return launch_pass(k, grid, g.threads, g.smem, st, a, (TW)tw, tiles, map, map2);
     } else {
         if constexpr (col_xstage<R, L>()) {
             if (g.persistent) {
@@ -396,17 +417,15 @@ inline cudaError_t col_launch_t(const ColArgs &a, int64_t tiles, const void *tw,
                 else memset(&map, 0, sizeof(map));
                 if (tmap2) map2 = *tmap2;
                 else memset(&map2, 0, sizeof(map2));
-                k<<<grid, g.threads, g.smem, st>>>(a, (TW)tw, tiles, map, map2);
-                return cudaGetLastError();
+                return launch_pass(k, grid, g.threads, g.smem, st, a, (TW)tw, tiles, map, map2);
             }
         }
         auto k = a.axis == 0 ? (a.inverse ? col_one_tile_kernel<R, L, 0, true>() : col_one_tile_kernel<R, L, 0, false>())
                              : (a.inverse ? col_one_tile_kernel<R, L, 1, true>() : col_one_tile_kernel<R, L, 1, false>());
         ColArgs b = a;
         b.pf_stride = col_l2_prefetch<R, L>(a.axis) ? persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) : 0;
-        k<<<(unsigned)tiles, g.threads, g.smem, st>>>(b, (TW)tw);
+        return launch_pass(k, tiles, g.threads, g.smem, st, b, (TW)tw);
     }
-    return cudaGetLastError();
 }
 
 template <typename R, int M>
@@ -416,16 +435,15 @@ inline cudaError_t zr2c_launch_t(const ZArgs &a, const void *tw, const void *rot
     z_geom_t<R, M>(&g);
     const int64_t blocks = (a.nlines + g.per_block - 1) / g.per_block;
     typedef const typename twvec<R>::T *TW;
-    if (a.max_blocks > 0 && blocks > a.max_blocks)
-        z_kernel<R, M, false, true, false>()<<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
-    else {
+    if (a.max_blocks > 0 && blocks > a.max_blocks) {
+        return launch_pass(z_kernel<R, M, false, true, false>(), a.max_blocks, g.threads, g.smem, st, a, (TW)tw, (TW)rot);
+    } else {
         const bool unit = a.scale_edge == 1.0 && a.scale_mid == 1.0;
         auto k = unit ? z_kernel<R, M, false, false, true>() : z_kernel<R, M, false, false, false>();
         ZArgs b = a;
         b.pf_lines = z_l2pf<R, M, false>() ? (int64_t)persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) * g.per_block : 0;
-        k<<<(unsigned)blocks, g.threads, g.smem, st>>>(b, (TW)tw, (TW)rot);
+        return launch_pass(k, blocks, g.threads, g.smem, st, b, (TW)tw, (TW)rot);
     }
-    return cudaGetLastError();
 }
 
 template <typename R, int M>
@@ -435,16 +453,15 @@ inline cudaError_t zc2r_launch_t(const ZArgs &a, const void *tw, const void *rot
     z_geom_t<R, M>(&g);
     const int64_t blocks = (a.nlines + g.per_block - 1) / g.per_block;
     typedef const typename twvec<R>::T *TW;
-    if (a.max_blocks > 0 && blocks > a.max_blocks)
-        z_kernel<R, M, true, true, false>()<<<(unsigned)a.max_blocks, g.threads, g.smem, st>>>(a, (TW)tw, (TW)rot);
-    else {
+    if (a.max_blocks > 0 && blocks > a.max_blocks) {
+        return launch_pass(z_kernel<R, M, true, true, false>(), a.max_blocks, g.threads, g.smem, st, a, (TW)tw, (TW)rot);
+    } else {
         const bool unit = fx_unit_scale(a.scale_mid);
         auto k = unit ? z_kernel<R, M, true, false, true>() : z_kernel<R, M, true, false, false>();
         ZArgs b = a;
         b.pf_lines = z_l2pf<R, M, true>() ? (int64_t)persistent_grid(k, g.threads, g.smem, (int64_t)1 << 40) * g.per_block : 0;
-        k<<<(unsigned)blocks, g.threads, g.smem, st>>>(b, (TW)tw, (TW)rot);
+        return launch_pass(k, blocks, g.threads, g.smem, st, b, (TW)tw, (TW)rot);
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- fused

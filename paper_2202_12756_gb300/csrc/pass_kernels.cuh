@@ -31,6 +31,19 @@
 
 namespace fft3d {
 
+// Start of every pass kernel: a pass is launched while the kernel before it on
+// the stream drains (launch_pass) and waits here until that kernel has
+// completed and its writes are visible.  All blocks wait, so completion
+// carries over from kernel to kernel.
+__device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// A block lets the next pass be launched when only its stores are left.  From
+// the start of the block instead, the next pass's blocks take the slots of the
+// first SMs that run dry and crowd there: 128^3 pair 31.8 -> 40.1 us.  The
+// persistent and the link-bound (max_blocks) kernels release nothing: a
+// waiting block would keep another stream's passes off the SM for long.
+// 256^3 float pair 151 -> 136 us, 64^3 double pair (each waited for) 78 -> 72.
+__device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 // ------------------------------------------------------------ layouts
 // Complex half-spectrum array, logically [N0][N1][M + 1].
 //   standard: main[(k0 N1 + k1) (M + 1) + k2]
@@ -98,7 +111,10 @@ template <typename C, int W> struct ColEx {
 // Which column lane c of tile t owns, and where it lives in the source and
 // destination layouts.  Lanes past the last column get the last column's
 // address (so every load is in bounds) and `false`: they compute on a copy
-// and store nothing.  Columns never mix, so this is harmless.
+// and store nothing.  Columns never mix, so this is harmless.  Tile numbers
+// and the columns of a field fit 32 bits, and 32-bit divisions take a fifth of
+// the instructions of 64-bit ones, which every thread would run for 8 to 24
+// elements.
 template <typename C, int W>
 __device__ __forceinline__ bool col_decode(const ColArgs &a, int64_t t, int c, C *&sp, int64_t &ss, C *&dp,
                                            int64_t &ds)
@@ -106,21 +122,21 @@ __device__ __forceinline__ bool col_decode(const ColArgs &a, int64_t t, int c, C
     int64_t k0 = 0, k1 = 0, k2 = 0;
     bool valid;
     if (a.axis == 0) {
-        const int64_t total = a.n1 * (a.m + 1);
-        const int64_t b = (uint32_t)t / (uint32_t)a.tiles_per_field;  // field of a batched plan (t < 2^32)
-        int64_t f = (t - b * a.tiles_per_field) * W + c;  // flat (k1, k2) index
+        const uint32_t m1 = (uint32_t)a.m + 1, total = (uint32_t)a.n1 * m1;
+        const uint32_t b = (uint32_t)t / (uint32_t)a.tiles_per_field;  // field of a batched plan
+        uint32_t f = ((uint32_t)t - b * (uint32_t)a.tiles_per_field) * W + c;  // flat (k1, k2) index
         valid = f < total;
         f = valid ? f : total - 1;
         k0 = b * a.n0;
-        k1 = f / (a.m + 1);
-        k2 = f - k1 * (a.m + 1);
+        k1 = f / m1;
+        k2 = f - (uint32_t)k1 * m1;
     } else if (a.nyq_in_plane) {
-        k0 = t / a.tiles_per_plane;
+        k0 = (uint32_t)t / (uint32_t)a.tiles_per_plane;
         k2 = (t - k0 * a.tiles_per_plane) * W + c;
         valid = k2 <= a.m;
         k2 = valid ? k2 : a.m;
     } else if (t < a.tiles_main) {
-        k0 = t / a.tiles_per_plane;
+        k0 = (uint32_t)t / (uint32_t)a.tiles_per_plane;
         k2 = (t - k0 * a.tiles_per_plane) * W + c;
         valid = k2 < a.m;
         k2 = valid ? k2 : a.m - 1;
@@ -200,6 +216,7 @@ __device__ __forceinline__ void col_tile(const ColArgs &a, int64_t tile, unsigne
     }
     ColEx<C, W> ex{(C *)smem, c};
     line_fft<R, L, E>(v, j, tw, ex);
+    pass_release();
     if (valid) {
         C *dj = dp + (int64_t)j * ds;
         const int64_t dstep = (int64_t)NT * ds;
@@ -218,6 +235,7 @@ __global__ void __launch_bounds__(W *(L / E))
 colpass_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pass_begin();
     const int64_t pf = a.pf_stride > 0 && blockIdx.x + a.pf_stride < gridDim.x ? blockIdx.x + a.pf_stride : -1;
     col_tile<R, L, E, W, false, INV>(a, blockIdx.x, smem_raw, tw, pf);
 }
@@ -340,6 +358,7 @@ colpass_pipe_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int6
     constexpr int RSE = stage_row_elems<C, W>();
     static_assert(L % (2 * kTmaBoxRows) == 0 && NT % 2 == 0 && (RSE * sizeof(C)) % 16 == 0, "staging layout");
     extern __shared__ __align__(1024) unsigned char pipe_smem_raw[];
+    pass_begin();
     C *stage = (C *)pipe_smem_raw;
     C *stage_odd = stage + L / 2 * W;  // mode 2: odd rows, W + 2 wide
     R *exbuf = (R *)(stage + stage_elems<C, W, L>());
@@ -374,7 +393,7 @@ colpass_pipe_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int6
                         x = (int)((tt - b * a.tiles_per_field) * W);
                         y0 = (int)(b * a.n0);
                     } else {            // [N0 N1][M+1]: plane k0, columns c0..
-                        const int64_t k0 = tt / a.tiles_per_plane;
+                        const int64_t k0 = (uint32_t)tt / (uint32_t)a.tiles_per_plane;
                         x = (int)((tt - k0 * a.tiles_per_plane) * W);
                         y0 = (int)(k0 * a.n1);
                     }
@@ -383,7 +402,7 @@ colpass_pipe_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int6
                         tma_load_2d(smem_u32(stage + b * kTmaBoxRows * W), &tmap, x, y0 + b * kTmaBoxRows, mb);
                 } else {
                     mbar_arrive_expect_tx(mb, (unsigned)(L / 2 * (2 * W + 2) * sizeof(C)) + a.stall_tx);
-                    const int64_t k0 = tt / a.tiles_per_plane;
+                    const int64_t k0 = (uint32_t)tt / (uint32_t)a.tiles_per_plane;
                     const int c0 = (int)((tt - k0 * a.tiles_per_plane) * W);
                     const int y0 = (int)(k0 * (a.n1 / 2));
 #pragma unroll
@@ -523,6 +542,7 @@ colpass_xstage_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, in
     static_assert(L % (2 * kTmaBoxRows) == 0 && NT % 2 == 0 && (RSE * sizeof(C)) % 16 == 0, "staging layout");
     static_assert(line_nstages(L, E) >= 2 && L * W <= stage_elems<C, W, L>(), "the exchange reuses the staging buffer");
     extern __shared__ __align__(1024) unsigned char xstage_smem_raw[];
+    pass_begin();
     C *stage = (C *)xstage_smem_raw;
     C *stage_odd = stage + L / 2 * W;  // mode 2: odd rows, W + 2 wide
     uint64_t *mbar = (uint64_t *)(stage + stage_elems<C, W, L>());
@@ -556,7 +576,7 @@ colpass_xstage_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, in
                         x = (int)((tt - b * a.tiles_per_field) * W);
                         y0 = (int)(b * a.n0);
                     } else {            // [N0 N1][M+1]: plane k0, columns c0..
-                        const int64_t k0 = tt / a.tiles_per_plane;
+                        const int64_t k0 = (uint32_t)tt / (uint32_t)a.tiles_per_plane;
                         x = (int)((tt - k0 * a.tiles_per_plane) * W);
                         y0 = (int)(k0 * a.n1);
                     }
@@ -565,7 +585,7 @@ colpass_xstage_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, in
                         tma_load_2d(smem_u32(stage + b * kTmaBoxRows * W), &tmap, x, y0 + b * kTmaBoxRows, mb);
                 } else {
                     mbar_arrive_expect_tx(mb, (unsigned)(L / 2 * (2 * W + 2) * sizeof(C)) + a.stall_tx);
-                    const int64_t k0 = tt / a.tiles_per_plane;
+                    const int64_t k0 = (uint32_t)tt / (uint32_t)a.tiles_per_plane;
                     const int c0 = (int)((tt - k0 * a.tiles_per_plane) * W);
                     const int y0 = (int)(k0 * (a.n1 / 2));
 #pragma unroll
@@ -792,6 +812,7 @@ colpass_pair_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int6
     static_assert(H * W * NT * sizeof(C) <= (size_t)split_rows<LH>() * W * sizeof(R), "receive buffer");
     static_assert(line_nstages(LH, E) >= 2, "the transform must end its exchange-buffer use on a barrier");
     extern __shared__ __align__(1024) unsigned char pair_smem_raw[];
+    pass_begin();
     C *stage = (C *)pair_smem_raw;  // [LH][W] or, odd rows of a.bulk = 2, [LH][W + 2]
     R *exbuf = (R *)(stage + LH * (W + 2));
     // mbarriers: the tile's staging copies, the partner's data, the partner's exchange buffer free
@@ -836,7 +857,7 @@ colpass_pair_kernel(ColArgs a, const typename twvec<R>::T *__restrict__ tw, int6
                     x = (int)((tt - b * a.tiles_per_field) * W);
                     y0 = (int)(b * (a.n0 / 2));
                 } else {
-                    const int64_t k0 = tt / a.tiles_per_plane;
+                    const int64_t k0 = (uint32_t)tt / (uint32_t)a.tiles_per_plane;
                     x = (int)((tt - k0 * a.tiles_per_plane) * W);
                     y0 = (int)(k0 * (a.n1 / 2));
                 }
@@ -1133,6 +1154,7 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
     if constexpr (FFT3D_ROTCONST && sizeof(R) == 4) rot_j = __ldg(rot + j);
 
     line_fft<R, M, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     C *out = (C *)a.cplx.main + (active ? line : 0) * (M + 1);
     const R se = R(a.scale_edge), sm = R(a.scale_mid);
@@ -1302,6 +1324,7 @@ __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsign
     }
 
     line_fft<R, M, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     const R s = R(sizeof(R) == 8 ? 2.0 * a.scale_mid : a.scale_mid);
     C *out = (C *)((R *)a.real_out + l * a.real_pitch);
@@ -1346,6 +1369,7 @@ __device__ __forceinline__ void zr2c_pairs(const ZArgs &a, int64_t line0, unsign
         v[i] = cmake<C>(act0 ? in0[n] : R(0), act1 ? in1[n] : R(0));
     }
     line_fft<R, N, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     constexpr bool LR = pad_linear_reads<P>(NT);
     constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
@@ -1428,6 +1452,7 @@ __device__ __forceinline__ void zc2r_pairs(const ZArgs &a, int64_t line0, unsign
         v[i] = cswap(cmake<C>(x0.x - x1.y, x0.y + x1.x));
     }
     line_fft<R, N, E>(v, j, tw, ex);
+    if (a.max_blocks == 0) pass_release();
 
     const R s = R(a.scale_mid);
     R *out0 = (R *)a.real_out + la * a.real_pitch;
