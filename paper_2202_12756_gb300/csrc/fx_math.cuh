@@ -1,7 +1,7 @@
 // 64-bit block fixed-point arithmetic for the double-precision transforms.
 //
-// GB300 issues two FP64 instructions per SM and clock, but 64 integer ones,
-// and a 32 x 32 + 64 -> 64 bit multiply-add (mad.wide) counts as one.  The
+// GB300 issues two FP64 instructions per SM and clock, but 64 integer ones
+// on each of two pipes, and about 28 multiplications 32 x 32 -> 64 bit.  The
 // FP64 passes were bound by FP64 issue (30 instructions per element, 15
 // clocks, against 1.5 clocks for the element's HBM traffic), so double lines
 // are transformed as integers instead: a line (or column) is scaled by one
@@ -52,18 +52,20 @@ __host__ __device__ constexpr int fx_stage_shift(int r) { return r <= 4 ? 2 : 1 
 FX_HD int32_t fx_lo(int64_t a) { return (int32_t)(uint32_t)a; }
 // high limb that goes with the low limb read as a signed number
 FX_HD int32_t fx_hi(int64_t a) { return (int32_t)((uint64_t)a >> 32) + (int32_t)((uint32_t)a >> 31); }
-// a b + c.  With variable factors the compiler is held to one mad.wide: where it
-// sees both sign extensions apart from the product, it multiplies 64 x 64 bits
-// (a product by a table twiddle took 54 instructions instead of 31).
-FX_HD int64_t fx_madk(int32_t a, int32_t b, int64_t c) { return (int64_t)a * b + c; }  // constant b
-FX_HD int64_t fx_mad(int32_t a, int32_t b, int64_t c)
+// a b as one mul.wide, whose sums with other products are 64-bit additions.
+// Measured on GB300 in registers, a complex product by a table twiddle takes 57
+// issue cycles of an SM quarter (21 instructions) this way, against 67 (31) as
+// mad.wide chains, which the compiler splits, and 54 instructions in plain C++,
+// which it turns into 64 x 64-bit products where it sees the sign extensions
+// apart from the multiplication.
+FX_HD int64_t fx_mul(int32_t a, int32_t b)
 {
 #ifdef __CUDA_ARCH__
     int64_t r;
-    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
     return r;
 #else
-    return (int64_t)a * b + c;
+    return (int64_t)a * b;
 #endif
 }
 
@@ -83,9 +85,9 @@ FX_HD fxc cmul(fxc z, fxtw w)
     const int32_t xl = fx_lo(z.x), xh = fx_hi(z.x), yl = fx_lo(z.y), yh = fx_hi(z.y);
     const int32_t nh = -w.yh, nl = -w.yl;
     const int64_t half = 0x80000000LL;
-    const int64_t mr = fx_mad(yl, nh, fx_mad(yh, nl, fx_mad(xl, w.xh, fx_mad(xh, w.xl, half))));
-    const int64_t mi = fx_mad(yl, w.xh, fx_mad(yh, w.xl, fx_mad(xl, w.yh, fx_mad(xh, w.yl, half))));
-    return fx_make(fx_mad(yh, nh, fx_mad(xh, w.xh, mr >> 32)), fx_mad(yh, w.xh, fx_mad(xh, w.yh, mi >> 32)));
+    const int64_t mr = fx_mul(yl, nh) + fx_mul(yh, nl) + fx_mul(xl, w.xh) + fx_mul(xh, w.xl) + half;
+    const int64_t mi = fx_mul(yl, w.xh) + fx_mul(yh, w.xl) + fx_mul(xl, w.yh) + fx_mul(xh, w.yl) + half;
+    return fx_make(fx_mul(yh, nh) + fx_mul(xh, w.xh) + (mr >> 32), fx_mul(yh, w.xh) + fx_mul(xh, w.yh) + (mi >> 32));
 }
 // z conj(w) 2^-d
 FX_HD fxc cmulc(fxc z, fxtw w)
@@ -174,8 +176,8 @@ template <int P> FX_HD fxc fx_rot96(fxc z)
                           nl = fx_limb_l(M.k), nh = fx_limb_h(M.k);
         const int32_t xl = fx_lo(z.x), xh = fx_hi(z.x), yl = fx_lo(z.y), yh = fx_hi(z.y);
         const int64_t half = 0x80000000LL;
-        const int64_t mr = fx_madk(yl, sh, fx_madk(yh, sl, fx_madk(xl, ch, fx_madk(xh, cl, half))));
-        const int64_t mi = fx_madk(xl, nh, fx_madk(xh, nl, fx_madk(yl, ch, fx_madk(yh, cl, half))));
+        const int64_t mr = fx_mul(yl, sh) + fx_mul(yh, sl) + fx_mul(xl, ch) + fx_mul(xh, cl) + half;
+        const int64_t mi = fx_mul(xl, nh) + fx_mul(xh, nl) + fx_mul(yl, ch) + fx_mul(yh, cl) + half;
         int64_t re = mr >> 32, im = mi >> 32;
         if constexpr (C.unit == 1) re += z.x, im += z.y;
         if constexpr (C.unit == -1) re -= z.x, im -= z.y;
@@ -183,7 +185,7 @@ template <int P> FX_HD fxc fx_rot96(fxc z)
         if constexpr (S.unit == -1) re -= z.y;
         if constexpr (M.unit == 1) im += z.x;
         if constexpr (M.unit == -1) im -= z.x;
-        return fx_make(fx_madk(yh, sh, fx_madk(xh, ch, re)), fx_madk(xh, nh, fx_madk(yh, ch, im)));
+        return fx_make(fx_mul(yh, sh) + fx_mul(xh, ch) + re, fx_mul(xh, nh) + fx_mul(yh, ch) + im);
     }
 }
 // a cos(2 pi P / 96) for a real a, |a| < 2^62 (0 < P <= 16)
@@ -193,7 +195,7 @@ template <int P> FX_HD int64_t fx_scale96(int64_t a)
     static_assert(C.unit == 1, "first eighth");
     constexpr int32_t cl = fx_limb_l(C.k), ch = fx_limb_h(C.k);
     const int32_t l = fx_lo(a), h = fx_hi(a);
-    return fx_mad(h, ch, a + (fx_mad(l, ch, fx_mad(h, cl, 0x80000000LL)) >> 32));
+    return a + fx_mul(h, ch) + ((fx_mul(l, ch) + fx_mul(h, cl) + 0x80000000LL) >> 32);
 }
 // z exp(-2 pi i / 8), z exp(-2 pi i 3 / 8)
 FX_HD fxc w8_1(fxc z) { return fx_make(fx_scale96<12>(z.x + z.y), fx_scale96<12>(z.y - z.x)); }
