@@ -27,7 +27,10 @@ __device__ __forceinline__ fxtw fx_ldg(const fxtw *p)
     return fxtw{q.x, q.y, q.z, q.w};
 }
 
-// Scale code of a thread's n complex values.
+// Scale code of a thread's n complex values.  (Bounding the L1 norm by twice the
+// larger component of each takes 17 issue cycles of an SM quarter per value
+// instead of 21, but a line with one large entry loses up to a bit: relative L2
+// error 2.4e-16 at 2048 points, above the FP64 transform's 2.1e-16.)
 template <int N> __device__ __forceinline__ int fx_thread_code(const double2 *v)
 {
     int32_t tm = 0;

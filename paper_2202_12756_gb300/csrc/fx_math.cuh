@@ -265,8 +265,14 @@ constexpr int kFxMinCode = 128, kFxMaxCode = 1900, kFxZeroCode = 1023;
 FX_HD float fx_mag(int32_t top, int32_t expo)  // |v| / 2^(expo's exponent), at least 2^-100
 {
     const int32_t fl = expo - (100 << 20);
-    const uint32_t t = (uint32_t)(top > fl ? top : fl);
-    return fx_float(t * 8u + ((127u << 20) - (uint32_t)expo) * 8u);
+    const uint32_t t = (uint32_t)(top > fl ? top : fl), off = ((127u << 20) - (uint32_t)expo) * 8u;
+#ifdef __CUDA_ARCH__
+    uint32_t b;
+    asm("mad.lo.u32 %0, %1, 8, %2;" : "=r"(b) : "r"(t), "r"(off));  // not on the pipe of the maxima
+    return fx_float(b);
+#else
+    return fx_float(t * 8u + off);
+#endif
 }
 FX_HD int fx_code(int32_t top_max, float sum)
 {
@@ -298,16 +304,17 @@ FX_HD int64_t fx_from(double v, int g, int bits)
 #endif
 }
 
-// Position of the leading bit of h that differs from its sign, -1 without one.
-FX_HD int32_t fx_lead(int32_t h)
+// Left shift that brings the leading bit of h that differs from its sign to bit
+// 31, -1 without one.
+FX_HD int32_t fx_lead_shift(int32_t h)
 {
 #ifdef __CUDA_ARCH__
-    int32_t p;
-    asm("bfind.s32 %0, %1;" : "=r"(p) : "r"(h));
-    return p;
+    int32_t n;
+    asm("bfind.shiftamt.s32 %0, %1;" : "=r"(n) : "r"(h));
+    return n;
 #else
     const uint32_t a = (uint32_t)(h ^ (h >> 31));
-    return a ? 31 - __builtin_clz(a) : -1;
+    return a ? __builtin_clz(a) : -1;
 #endif
 }
 FX_HD uint32_t fx_shl_hi(uint32_t lo, uint32_t hi, uint32_t n)  // high word of hi:lo << n, n < 32
@@ -320,19 +327,21 @@ FX_HD uint32_t fx_shl_hi(uint32_t lo, uint32_t hi, uint32_t n)  // high word of 
 }
 
 // X 2^e, rounded to nearest (ties towards +infinity, so that they leave no
-// bias), for |X| < 2^62 and e in [-1000, 900], on the integer pipe.  Serves
-// |X| >= 2^32, else clears the sign bit of `big` and returns anything.
+// bias), for |X| < 2^62 and e in [-1000, 900], on the integer pipes.  Serves
+// |X| >= 2^32, else clears the sign bit of `big` and returns anything.  The
+// exponent is a product by 2^20, which the multiply pipe takes off the adders
+// (42 issue cycles of an SM quarter per complex value, 49 with shifts).
 FX_HD double fx_to_big(int64_t X, int e, int32_t &big)
 {
     const uint32_t hi = (uint32_t)((uint64_t)X >> 32), lo = (uint32_t)(uint64_t)X;
     const uint32_t s = (uint32_t)((int32_t)hi >> 31);
-    const int32_t p = fx_lead((int32_t)hi);
-    big &= ~p;
-    const uint32_t n = (uint32_t)(30 - p) & 31;
+    const int32_t n1 = fx_lead_shift((int32_t)hi);
+    big &= ~n1;
+    const uint32_t n = (uint32_t)n1 - 1;
     // |X| 2^n with its leading bit at 62 (one less in the last place if X < 0)
-    const uint64_t v = ((uint64_t)(fx_shl_hi(lo, hi, n) ^ s) << 32 | ((lo << n) ^ s)) + 512;
-    const uint32_t r = (uint32_t)(v >> 42) + ((uint32_t)p << 20);
-    return fx_double((uint64_t)(r + (((uint32_t)(e + 1054) << 20) | (s & 0x80000000u))) << 32 | (uint32_t)(v >> 10));
+    const uint64_t v = ((uint64_t)(fx_shl_hi(lo, hi, n & 31) ^ s) << 32 | ((lo << (n & 31)) ^ s)) + 512;
+    const uint32_t r = (uint32_t)(v >> 42) + (((uint32_t)(e + 1084) << 20) - n * 1048576u);
+    return fx_double((uint64_t)(r | (s & 0x80000000u)) << 32 | (uint32_t)(v >> 10));
 }
 // The same for any |X| < 2^62, with two FP64 additions (ties to even).
 FX_HD double fx_to(int64_t X, int e)
