@@ -153,7 +153,7 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
     }
     ColEx<fxc, W> ex{(fxc *)smem_raw, c};
     line_fft<fx64, L, E>(v, j, tw, ex);
-    pass_release();
+    pass_release<double, E>();
     const int e = g - 1023 - kFxBits + fx_line_shift<L, E>();
     if (valid) {
         double2 *dj = dp + (int64_t)j * ds;
@@ -232,7 +232,7 @@ __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, uns
         for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
     }
     line_fft<fx64, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<double, E>();
 
     const int e = g - 1023 - kFxBits + fx_line_shift<M, E>();
     double2 *out = (double2 *)a.cplx.main + (active ? line : 0) * (M + 1);
@@ -374,7 +374,7 @@ __device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, uns
         ex.sync();
     }
     line_fft<fx64, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<double, E>();
 
     int e = g - 1023 - (kFxBits - 2) + fx_line_shift<M, E>();
     const double f = fx_split_scale<UNIT>(a.scale_mid, e);
@@ -418,7 +418,7 @@ __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, uns
         for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
     }
     line_fft<fx64, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<double, E>();
 
     constexpr bool LR = pad_linear_reads<P>(NT);
     constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
@@ -514,7 +514,7 @@ __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, uns
         ex.sync();
     }
     line_fft<fx64, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<double, E>();
 
     int e = g - 1023 - (kFxBits - 1) + fx_line_shift<N, E>();
     const double f = fx_split_scale<UNIT>(a.scale_mid, e);

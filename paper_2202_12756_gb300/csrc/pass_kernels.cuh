@@ -42,7 +42,12 @@ __device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.wait
 // persistent and the link-bound (max_blocks) kernels release nothing: a
 // waiting block would keep another stream's passes off the SM for long.
 // 256^3 float pair 151 -> 136 us, 64^3 double pair (each waited for) 78 -> 72.
-__device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+// Float threads of 24 elements release nothing either: their kernels are at the
+// edge of their register budgets (the 768-point R2C one went 120 -> 154).
+template <typename R, int E> __device__ __forceinline__ void pass_release()
+{
+    if constexpr (!(sizeof(R) == 4 && E == 24)) asm volatile("griddepcontrol.launch_dependents;\n");
+}
 
 // ------------------------------------------------------------ layouts
 // Complex half-spectrum array, logically [N0][N1][M + 1].
@@ -216,7 +221,7 @@ __device__ __forceinline__ void col_tile(const ColArgs &a, int64_t tile, unsigne
     }
     ColEx<C, W> ex{(C *)smem, c};
     line_fft<R, L, E>(v, j, tw, ex);
-    pass_release();
+    pass_release<R, E>();
     if (valid) {
         C *dj = dp + (int64_t)j * ds;
         const int64_t dstep = (int64_t)NT * ds;
@@ -1154,7 +1159,7 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
     if constexpr (FFT3D_ROTCONST && sizeof(R) == 4) rot_j = __ldg(rot + j);
 
     line_fft<R, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<R, E>();
 
     C *out = (C *)a.cplx.main + (active ? line : 0) * (M + 1);
     const R se = R(a.scale_edge), sm = R(a.scale_mid);
@@ -1324,7 +1329,7 @@ __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsign
     }
 
     line_fft<R, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<R, E>();
 
     const R s = R(sizeof(R) == 8 ? 2.0 * a.scale_mid : a.scale_mid);
     C *out = (C *)((R *)a.real_out + l * a.real_pitch);
@@ -1369,7 +1374,7 @@ __device__ __forceinline__ void zr2c_pairs(const ZArgs &a, int64_t line0, unsign
         v[i] = cmake<C>(act0 ? in0[n] : R(0), act1 ? in1[n] : R(0));
     }
     line_fft<R, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<R, E>();
 
     constexpr bool LR = pad_linear_reads<P>(NT);
     constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
@@ -1452,7 +1457,7 @@ __device__ __forceinline__ void zc2r_pairs(const ZArgs &a, int64_t line0, unsign
         v[i] = cswap(cmake<C>(x0.x - x1.y, x0.y + x1.x));
     }
     line_fft<R, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release();
+    if (a.max_blocks == 0) pass_release<R, E>();
 
     const R s = R(a.scale_mid);
     R *out0 = (R *)a.real_out + la * a.real_pitch;
