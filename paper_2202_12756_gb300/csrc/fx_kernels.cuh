@@ -5,8 +5,9 @@
 // double range) runs the FP64 pass instead, from the same twiddle tables.
 //
 // Measured on GB300 in place (FP64 arithmetic -> fixed point): 1024^3 pair
-// 190.1 -> 36 ms, 512^3 21.6 -> 4.1 ms; relative L2 error of one transform
-// 2.0-2.6e-16 -> 0.8-1.6e-16 against quadruple precision over every line length.
+// 190.1 -> 31.8 ms, 512^3 21.6 -> 3.54 ms; relative L2 error of one transform
+// against extended precision, over line lengths, noise and single-spike lines:
+// 1.6-2.8e-16 -> 0.5-1.8e-16.
 #pragma once
 
 #include "pass_kernels.cuh"

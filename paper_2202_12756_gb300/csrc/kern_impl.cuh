@@ -82,7 +82,7 @@ constexpr int kPairW = 16;  // columns of a CTA-pair tile (128-byte float rows)
 // 64 registers a thread, so 1024 threads an SM hide the latencies of the
 // integer pipe that 512 threads of 16 elements leave open, and a small grid
 // finishes sooner.  Measured on GB300: 512^3 y-pass 0.78 -> 0.64 ms, 64^3 pair
-// 71 -> 55 us; at 1024 points (a third exchange, 512-thread blocks) 6.1 -> 6.7 ms.
+// 71 -> 55 us; at 1024 points (a third exchange, 512-thread blocks) 5.5 -> 6.0 ms.
 template <typename R, int L> __host__ __device__ constexpr int col_E()
 {
     return col_pipe<R, L>() ? 32 : ((sizeof(R) == 8 && is_pow2(L) && L >= 8 && L <= 512) ? 8 : line_E(L));
