@@ -157,6 +157,19 @@ __host__ __device__ constexpr int32_t fx_limb_h(int64_t k)
     return (int32_t)((k >> 32) + (int64_t)((uint64_t)k >> 31 & 1));
 }
 
+// a cos(2 pi P / 96) for a real a, |a| < 2^62 (0 < P <= 16)
+template <int P> FX_HD int64_t fx_scale96(int64_t a)
+{
+    constexpr FxConst C = fx_cos96(P);
+    static_assert(C.unit == 1, "first eighth");
+    constexpr int32_t cl = fx_limb_l(C.k), ch = fx_limb_h(C.k);
+    const int32_t l = fx_lo(a), h = fx_hi(a);
+    return a + fx_mul(h, ch) + ((fx_mul(l, ch) + fx_mul(h, cl) + 0x80000000LL) >> 32);
+}
+// z exp(-2 pi i / 8), z exp(-2 pi i 3 / 8)
+FX_HD fxc w8_1(fxc z) { return fx_make(fx_scale96<12>(z.x + z.y), fx_scale96<12>(z.y - z.x)); }
+FX_HD fxc w8_3(fxc z) { return fx_make(fx_scale96<12>(z.y - z.x), -fx_scale96<12>(z.x + z.y)); }
+
 // z exp(-2 pi i P / 96) at full scale, for |z| < 2^61
 template <int P> FX_HD fxc fx_rot96(fxc z)
 {
@@ -169,6 +182,21 @@ template <int P> FX_HD fxc fx_rot96(fxc z)
         return fx_make(-z.x, -z.y);
     } else if constexpr (p == 72) {
         return fx_make(-z.y, z.x);
+    } else if constexpr (p == 12) {
+        return w8_1(z);
+    } else if constexpr (p == 36) {
+        return w8_3(z);
+    } else if constexpr (p % 8 == 0 && p < 48) {
+        // 30, 60, 120, 150 degrees: a half, and one product by sin 60 per component
+        // (6 mul.wide instead of 12; with the 45 degrees above, 768^3 pair 15.4 -> 15.1 ms)
+        const int64_t hx = (z.x + 1) >> 1, hy = (z.y + 1) >> 1, sx = fx_scale96<8>(z.x), sy = fx_scale96<8>(z.y);
+        if constexpr (p == 8) return fx_make(sx + hy, sy - hx);
+        else if constexpr (p == 16) return fx_make(hx + sy, hy - sx);
+        else if constexpr (p == 32) return fx_make(sy - hx, -sx - hy);
+        else return fx_make(hy - sx, -sy - hx);
+    } else if constexpr (p > 48 && p % 4 == 0) {
+        const fxc r = fx_rot96<p - 48>(z);
+        return fx_make(-r.x, -r.y);
     } else {
         constexpr FxConst C = fx_cos96(p), S = fx_cos96(p - 24), M = fx_neg(fx_cos96(p - 24));
         // re = C x + S y, im = C y - S x
@@ -188,19 +216,6 @@ template <int P> FX_HD fxc fx_rot96(fxc z)
         return fx_make(fx_mul(yh, sh) + fx_mul(xh, ch) + re, fx_mul(xh, nh) + fx_mul(yh, ch) + im);
     }
 }
-// a cos(2 pi P / 96) for a real a, |a| < 2^62 (0 < P <= 16)
-template <int P> FX_HD int64_t fx_scale96(int64_t a)
-{
-    constexpr FxConst C = fx_cos96(P);
-    static_assert(C.unit == 1, "first eighth");
-    constexpr int32_t cl = fx_limb_l(C.k), ch = fx_limb_h(C.k);
-    const int32_t l = fx_lo(a), h = fx_hi(a);
-    return a + fx_mul(h, ch) + ((fx_mul(l, ch) + fx_mul(h, cl) + 0x80000000LL) >> 32);
-}
-// z exp(-2 pi i / 8), z exp(-2 pi i 3 / 8)
-FX_HD fxc w8_1(fxc z) { return fx_make(fx_scale96<12>(z.x + z.y), fx_scale96<12>(z.y - z.x)); }
-FX_HD fxc w8_3(fxc z) { return fx_make(fx_scale96<12>(z.y - z.x), -fx_scale96<12>(z.x + z.y)); }
-
 // ------------------------------------------------------------ double <-> fixed point
 FX_HD uint64_t fx_bits(double v)
 {
