@@ -28,22 +28,6 @@ __device__ __forceinline__ fxtw fx_ldg(const fxtw *p)
     return fxtw{q.x, q.y, q.z, q.w};
 }
 
-// Scale code of a thread's n complex values.  (Bounding the L1 norm by twice the
-// larger component of each takes 17 issue cycles of an SM quarter per value
-// instead of 21, but a line with one large entry loses up to a bit: relative L2
-// error 2.4e-16 at 2048 points, above the FP64 transform's 2.1e-16.)
-template <int N> __device__ __forceinline__ int fx_thread_code(const double2 *v)
-{
-    int32_t tm = 0;
-#pragma unroll
-    for (int i = 0; i < N; ++i) tm = max(tm, max(fx_top(v[i].x), fx_top(v[i].y)));
-    const int32_t ex = tm & 0x7ff00000;
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < N; ++i) s += fx_mag(fx_top(v[i].x), ex) + fx_mag(fx_top(v[i].y), ex);
-    return fx_code(tm, s);
-}
-
 // A complex result: by integer operations, or where a component is below 2^32
 // (2^-29 of the line's scale) or zero, by FP64 additions.
 __device__ __forceinline__ double2 fx_out(fxc z, int e)

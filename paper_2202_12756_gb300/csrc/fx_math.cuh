@@ -271,9 +271,10 @@ FX_HD int32_t fx_top(double v) { return (int32_t)((uint32_t)(fx_bits(v) >> 32) &
 
 // Scale of a line.  A thread gathers the largest `top` of its values, then
 // their sum as floats relative to that one's exponent; the scale code g (the
-// biased exponent of a power of two above the L1 norm; 0 for all zeros, kFxBad
-// with a non-finite value) is combined by max over the line.
-constexpr int kFxBad = 1 << 20;
+// biased exponent of a power of two above the L1 norm; 0 for all zeros, kFxTiny
+// for values whose tops are zeros, kFxBad with a non-finite value) is combined by
+// max over the line.
+constexpr int kFxBad = 1 << 20, kFxTiny = 1;
 // codes outside [kFxMinCode, kFxMaxCode] leave the exponent range of the conversions
 constexpr int kFxMinCode = 128, kFxMaxCode = 1900, kFxZeroCode = 1023;
 
@@ -295,6 +296,28 @@ FX_HD int fx_code(int32_t top_max, float sum)
     // (1 + 2^-12): mantissas were cut to 20 bits, the sum rounded
     const uint32_t s = fx_float_bits(sum * 1.000244140625f);
     return top_max == 0 ? 0 : (top_max >> 20) + (int)(s >> 23) - 126;
+}
+
+// Scale code of a thread's n complex values.  (Bounding the L1 norm by twice the
+// larger component of each takes 17 issue cycles of an SM quarter per value
+// instead of 21, but a line with one large entry loses up to a bit: relative L2
+// error 2.4e-16 at 2048 points, above the FP64 transform's 2.1e-16.)
+template <int N> FX_HD int fx_thread_code(const double2 *v)
+{
+    int32_t tm = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) tm = max(tm, max(fx_top(v[i].x), fx_top(v[i].y)));
+    if (tm == 0) {  // zeros, or values below 2^-1042, whose low words alone are set
+        uint64_t low = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) low |= fx_bits(v[i].x) | fx_bits(v[i].y);
+        return low << 1 ? kFxTiny : 0;
+    }
+    const int32_t ex = tm & 0x7ff00000;
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s += fx_mag(fx_top(v[i].x), ex) + fx_mag(fx_top(v[i].y), ex);
+    return fx_code(tm, s);
 }
 
 FX_HD bool fx_code_ok(int g) { return g == 0 || (g >= kFxMinCode && g <= kFxMaxCode); }
