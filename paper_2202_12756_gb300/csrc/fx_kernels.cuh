@@ -61,6 +61,16 @@ template <bool UNIT> __device__ __forceinline__ double2 fx_scale(double2 z, doub
     else return cscale(z, f);
 }
 
+// A block lets the next pass be launched when only its stores are left.  From
+// the start of the block instead, the next pass's blocks take the slots of the
+// first SMs that run dry and crowd there (128^3 float pair 31.8 -> 40.1 us).
+// The link-bound (max_blocks) kernels release nothing: a waiting block would
+// keep another stream's passes off the SM for long.  64^3 double pair, each
+// waited for: 78 -> 72 us.  The float passes release nothing either, as it
+// costs every block: 16-thread tiles of short columns 23 -> 39 us at
+// 4 x 1024 x 1024, where leaving it out costs the other grids nothing.
+__device__ __forceinline__ void pass_release() { asm volatile("griddepcontrol.launch_dependents;\n"); }
+
 // ------------------------------------------------------------ columns
 // Load of a column entry, asking L2 for the whole 128-byte line: the tile beside
 // it, run at the same time by another SM, wants the rest of it (512^3: y-pass
@@ -138,7 +148,7 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
     }
     ColEx<fxc, W> ex{(fxc *)smem_raw, c};
     line_fft<fx64, L, E>(v, j, tw, ex);
-    pass_release<double, E>();
+    pass_release();
     const int e = g - 1023 - kFxBits + fx_line_shift<L, E>();
     if (valid) {
         double2 *dj = dp + (int64_t)j * ds;
@@ -217,7 +227,7 @@ __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, uns
         for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
     }
     line_fft<fx64, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<double, E>();
+    if (a.max_blocks == 0) pass_release();
 
     const int e = g - 1023 - kFxBits + fx_line_shift<M, E>();
     double2 *out = (double2 *)a.cplx.main + (active ? line : 0) * (M + 1);
@@ -359,7 +369,7 @@ __device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, uns
         ex.sync();
     }
     line_fft<fx64, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<double, E>();
+    if (a.max_blocks == 0) pass_release();
 
     int e = g - 1023 - (kFxBits - 2) + fx_line_shift<M, E>();
     const double f = fx_split_scale<UNIT>(a.scale_mid, e);
@@ -403,7 +413,7 @@ __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, uns
         for (int i = 0; i < E; ++i) v[i] = fx_make(fx_from(r[i].x, g, kFxBits), fx_from(r[i].y, g, kFxBits));
     }
     line_fft<fx64, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<double, E>();
+    if (a.max_blocks == 0) pass_release();
 
     constexpr bool LR = pad_linear_reads<P>(NT);
     constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
@@ -499,7 +509,7 @@ __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, uns
         ex.sync();
     }
     line_fft<fx64, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<double, E>();
+    if (a.max_blocks == 0) pass_release();
 
     int e = g - 1023 - (kFxBits - 1) + fx_line_shift<N, E>();
     const double f = fx_split_scale<UNIT>(a.scale_mid, e);

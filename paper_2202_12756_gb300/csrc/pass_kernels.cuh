@@ -32,22 +32,10 @@
 namespace fft3d {
 
 // Start of every pass kernel: a pass is launched while the kernel before it on
-// the stream drains (launch_pass) and waits here until that kernel has
-// completed and its writes are visible.  All blocks wait, so completion
+// the stream ends (launch_pass; earlier where that one releases it) and waits
+// here until that kernel has completed and its writes are visible.  All blocks wait, so completion
 // carries over from kernel to kernel.
 __device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-// A block lets the next pass be launched when only its stores are left.  From
-// the start of the block instead, the next pass's blocks take the slots of the
-// first SMs that run dry and crowd there: 128^3 pair 31.8 -> 40.1 us.  The
-// persistent and the link-bound (max_blocks) kernels release nothing: a
-// waiting block would keep another stream's passes off the SM for long.
-// 256^3 float pair 151 -> 136 us, 64^3 double pair (each waited for) 78 -> 72.
-// Float threads of 24 elements release nothing either: their kernels are at the
-// edge of their register budgets (the 768-point R2C one went 120 -> 154).
-template <typename R, int E> __device__ __forceinline__ void pass_release()
-{
-    if constexpr (!(sizeof(R) == 4 && E == 24)) asm volatile("griddepcontrol.launch_dependents;\n");
-}
 
 // ------------------------------------------------------------ layouts
 // Complex half-spectrum array, logically [N0][N1][M + 1].
@@ -221,7 +209,6 @@ __device__ __forceinline__ void col_tile(const ColArgs &a, int64_t tile, unsigne
     }
     ColEx<C, W> ex{(C *)smem, c};
     line_fft<R, L, E>(v, j, tw, ex);
-    pass_release<R, E>();
     if (valid) {
         C *dj = dp + (int64_t)j * ds;
         const int64_t dstep = (int64_t)NT * ds;
@@ -1159,7 +1146,6 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
     if constexpr (FFT3D_ROTCONST && sizeof(R) == 4) rot_j = __ldg(rot + j);
 
     line_fft<R, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<R, E>();
 
     C *out = (C *)a.cplx.main + (active ? line : 0) * (M + 1);
     const R se = R(a.scale_edge), sm = R(a.scale_mid);
@@ -1329,7 +1315,6 @@ __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsign
     }
 
     line_fft<R, M, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<R, E>();
 
     const R s = R(sizeof(R) == 8 ? 2.0 * a.scale_mid : a.scale_mid);
     C *out = (C *)((R *)a.real_out + l * a.real_pitch);
@@ -1374,7 +1359,6 @@ __device__ __forceinline__ void zr2c_pairs(const ZArgs &a, int64_t line0, unsign
         v[i] = cmake<C>(act0 ? in0[n] : R(0), act1 ? in1[n] : R(0));
     }
     line_fft<R, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<R, E>();
 
     constexpr bool LR = pad_linear_reads<P>(NT);
     constexpr bool LREV = P < 0 || NT % (1 << P) == 0;
@@ -1457,7 +1441,6 @@ __device__ __forceinline__ void zc2r_pairs(const ZArgs &a, int64_t line0, unsign
         v[i] = cswap(cmake<C>(x0.x - x1.y, x0.y + x1.x));
     }
     line_fft<R, N, E>(v, j, tw, ex);
-    if (a.max_blocks == 0) pass_release<R, E>();
 
     const R s = R(a.scale_mid);
     R *out0 = (R *)a.real_out + la * a.real_pitch;
