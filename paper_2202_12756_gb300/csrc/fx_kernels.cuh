@@ -523,75 +523,55 @@ __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, uns
 }
 
 // A group of LPB lines, by the form that serves the length.
-template <typename R, int M, int E, int LPB, bool PF, bool UNIT>
-__device__ __forceinline__ void zr2c_group(const ZArgs &a, int64_t line0, unsigned char *smem,
-                                           const typename twvec<R>::T *__restrict__ tw,
-                                           const typename twvec<R>::T *__restrict__ rot)
+template <int M, int E, int LPB, bool UNIT>
+__device__ __forceinline__ void zr2c_fx_group(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                              const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
 {
-    if constexpr (!z_fixed<R, M>()) zr2c_lines<R, M, E, LPB, PF>(a, line0, smem, tw, rot);
-    else if constexpr (z_paired<R, M>()) zr2c_fx_pairs<M, E, LPB, UNIT>(a, line0, smem, tw);
+    if constexpr (z_paired<double, M>()) zr2c_fx_pairs<M, E, LPB, UNIT>(a, line0, smem, tw);
     else zr2c_fx_lines<M, E, LPB, UNIT>(a, line0, smem, tw, rot);
 }
-template <typename R, int M, int E, int LPB, bool PF, bool UNIT>
-__device__ __forceinline__ void zc2r_group(const ZArgs &a, int64_t line0, unsigned char *smem,
-                                           const typename twvec<R>::T *__restrict__ tw,
-                                           const typename twvec<R>::T *__restrict__ rot)
+template <int M, int E, int LPB, bool UNIT>
+__device__ __forceinline__ void zc2r_fx_group(const ZArgs &a, int64_t line0, unsigned char *smem,
+                                              const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
 {
-    if constexpr (!z_fixed<R, M>()) zc2r_lines<R, M, E, LPB, false, PF>(a, line0, smem, tw, rot);
-    else if constexpr (z_paired<R, M>()) zc2r_fx_pairs<M, E, LPB, UNIT>(a, line0, smem, tw);
+    if constexpr (z_paired<double, M>()) zc2r_fx_pairs<M, E, LPB, UNIT>(a, line0, smem, tw);
     else zc2r_fx_lines<M, E, LPB, UNIT>(a, line0, smem, tw, rot);
 }
 
-// One group of LPB lines per block; with LOOP, a grid of a.max_blocks blocks
-// walks the line groups (the host-memory form, bound by the CPU-GPU link).
-// Two instances because the loop slows the one-pass form down (up to 20%
-// measured for the C2R lines on GB300).
-// Minimum resident blocks in the launch bounds of the R2C z kernel: 1 (an
-// explicit floor, which changes the compiler's register budget) for float
-// lines of 3 * 2^k >= 384 points, else 0 (no floor).  Measured on GB300 the
-// floor cuts registers 127 -> 107 (M = 768) and 123 -> 95 (M = 384), and
-// the pass time by 7-8% (1536^3: 5.77 -> 5.33 ms); for M = 96 it is 1%
-// slower, and for the C2R kernel, or powers of two, it raises registers.
-template <typename R, int M, int E> __host__ __device__ constexpr int zr2c_minb()
-{
-    return sizeof(R) == 4 && E == 24 && M >= 384 ? 1 : 0;
-}
-template <typename R, int M, int E, int LPB> __host__ __device__ constexpr int fx_z_minb()
-{
-    return z_fixed<R, M>() ? fx_min_blocks(E, LPB * (M / E)) : 0;
-}
-
-template <typename R, int M, int E, int LPB, bool LOOP, bool UNIT>
-__global__ void __launch_bounds__(LPB *(M / E), sizeof(R) == 8 ? fx_z_minb<R, M, E, LPB>() : zr2c_minb<R, M, E>())
-zpass_r2c_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
-                 const typename twvec<R>::T *__restrict__ rot)
+// The z-passes in fixed point, blocks and LOOP as in zpass_r2c_kernel.  `a` is
+// __grid_constant__ because the slow path takes its address (without, every
+// thread copies it to local memory); the other z kernels are not: it costs
+// them registers (float R2C lines of 512 points 64 -> 80, 768-point looping
+// C2R ones 128 -> 159).
+template <int M, int E, int LPB, bool LOOP, bool UNIT>
+__global__ void __launch_bounds__(LPB *(M / E), fx_min_blocks(E, LPB *(M / E)))
+zpass_r2c_fx_kernel(const __grid_constant__ ZArgs a, const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pass_begin();
     if constexpr (LOOP) {
         for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
             if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
-            zr2c_group<R, M, E, LPB, false, false>(a, blk * LPB, smem_raw, tw, rot);
+            zr2c_fx_group<M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
         }
     } else {
-        zr2c_group<R, M, E, LPB, z_l2pf<R, M, false>(), UNIT>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+        zr2c_fx_group<M, E, LPB, UNIT>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
     }
 }
 
-template <typename R, int M, int E, int LPB, bool LOOP, bool UNIT>
-__global__ void __launch_bounds__(LPB *(M / E), fx_z_minb<R, M, E, LPB>())
-zpass_c2r_kernel(const __grid_constant__ ZArgs a, const typename twvec<R>::T *__restrict__ tw,
-                 const typename twvec<R>::T *__restrict__ rot)
+template <int M, int E, int LPB, bool LOOP, bool UNIT>
+__global__ void __launch_bounds__(LPB *(M / E), fx_min_blocks(E, LPB *(M / E)))
+zpass_c2r_fx_kernel(const __grid_constant__ ZArgs a, const fxtw *__restrict__ tw, const fxtw *__restrict__ rot)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pass_begin();
     if constexpr (LOOP) {
         for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
             if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
-            zc2r_group<R, M, E, LPB, false, false>(a, blk * LPB, smem_raw, tw, rot);
+            zc2r_fx_group<M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
         }
     } else {
-        zc2r_group<R, M, E, LPB, z_l2pf<R, M, true>(), UNIT>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+        zc2r_fx_group<M, E, LPB, UNIT>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
     }
 }
 

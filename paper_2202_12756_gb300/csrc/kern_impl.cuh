@@ -234,13 +234,14 @@ template <typename R, int L> inline cudaError_t col_prepare_t()
     }
 }
 
-// z kernels of a length: [LOOP, UNIT]; UNIT only for double lines without LOOP.
+// z kernels of a length; UNIT (never with LOOP) makes a difference to fixed-point lines only.
 template <typename R, int M, bool C2R, bool LOOP, bool UNIT> inline auto z_kernel()
 {
     constexpr int E = z_E<R, M>(), LPB = z_LPB<R, M>();
-    constexpr bool U = UNIT && z_fixed<R, M>();
-    if constexpr (C2R) return zpass_c2r_kernel<R, M, E, LPB, LOOP, U>;
-    else return zpass_r2c_kernel<R, M, E, LPB, LOOP, U>;
+    if constexpr (!z_fixed<R, M>() && C2R) return zpass_c2r_kernel<R, M, E, LPB, LOOP>;
+    else if constexpr (!z_fixed<R, M>()) return zpass_r2c_kernel<R, M, E, LPB, LOOP>;
+    else if constexpr (C2R) return zpass_c2r_fx_kernel<M, E, LPB, LOOP, UNIT>;
+    else return zpass_r2c_fx_kernel<M, E, LPB, LOOP, UNIT>;
 }
 
 template <typename R, int M> inline cudaError_t z_prepare_t()

@@ -1453,4 +1453,51 @@ __device__ __forceinline__ void zc2r_pairs(const ZArgs &a, int64_t line0, unsign
     }
 }
 
+// One group of LPB lines per block; with LOOP, a grid of a.max_blocks blocks
+// walks the line groups (the host-memory form, bound by the CPU-GPU link).
+// Two instances because the loop slows the one-pass form down (up to 20%
+// measured for the C2R lines on GB300).
+// Minimum resident blocks in the launch bounds of the R2C z kernel: 1 (an
+// explicit floor, which changes the compiler's register budget) for float
+// lines of 3 * 2^k >= 384 points, else 0 (no floor).  Measured on GB300 the
+// floor cuts registers 127 -> 107 (M = 768) and 123 -> 95 (M = 384), and
+// the pass time by 7-8% (1536^3: 5.77 -> 5.33 ms); for M = 96 it is 1%
+// slower, and for the C2R kernel, or powers of two, it raises registers.
+template <typename R, int M, int E> __host__ __device__ constexpr int zr2c_minb()
+{
+    return sizeof(R) == 4 && E == 24 && M >= 384 ? 1 : 0;
+}
+
+template <typename R, int M, int E, int LPB, bool LOOP>
+__global__ void __launch_bounds__(LPB *(M / E), zr2c_minb<R, M, E>())
+zpass_r2c_kernel(ZArgs a, const typename twvec<R>::T *__restrict__ tw, const typename twvec<R>::T *__restrict__ rot)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pass_begin();
+    if constexpr (LOOP) {
+        for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
+            if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
+            zr2c_lines<R, M, E, LPB>(a, blk * LPB, smem_raw, tw, rot);
+        }
+    } else {
+        zr2c_lines<R, M, E, LPB, z_l2pf<R, M, false>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+    }
+}
+
+template <typename R, int M, int E, int LPB, bool LOOP>
+__global__ void __launch_bounds__(LPB *(M / E))
+zpass_c2r_kernel(ZArgs a, const typename twvec<R>::T *__restrict__ tw, const typename twvec<R>::T *__restrict__ rot)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pass_begin();
+    if constexpr (LOOP) {
+        for (int64_t blk = blockIdx.x; blk * LPB < a.nlines; blk += gridDim.x) {
+            if (blk != blockIdx.x) __syncthreads();  // shared memory free for the next line group
+            zc2r_lines<R, M, E, LPB, false>(a, blk * LPB, smem_raw, tw, rot);
+        }
+    } else {
+        zc2r_lines<R, M, E, LPB, false, z_l2pf<R, M, true>()>(a, (int64_t)blockIdx.x * LPB, smem_raw, tw, rot);
+    }
+}
+
 }  // namespace fft3d
