@@ -19,9 +19,6 @@ namespace fft3d {
 template <typename R, int L> __host__ __device__ constexpr bool col_fixed() { return sizeof(R) == 8 && L >= 8; }
 template <typename R, int M> __host__ __device__ constexpr bool z_fixed() { return sizeof(R) == 8 && M >= 4; }
 
-// table scale of the R2C rotation factors
-constexpr int kFxRotShift = 2;
-
 __device__ __forceinline__ fxtw fx_ldg(const fxtw *p)
 {
     const int4 q = __ldg((const int4 *)p);

@@ -46,6 +46,8 @@ struct __align__(16) fxtw {
 // values stay below 2^kFxBits in magnitude
 constexpr int kFxBits = 61;
 
+// table scale of the R2C rotation factors
+constexpr int kFxRotShift = 2;
 // scale 2^-D of the twiddles that go with a radix-r butterfly (r > 1)
 __host__ __device__ constexpr int fx_stage_shift(int r) { return r <= 4 ? 2 : 1 + fx_stage_shift((r + 1) / 2); }
 
@@ -455,10 +457,15 @@ FX_HD fxtw fx_twiddle(uint32_t p, uint32_t d, int shift)
     fx_limbs((-s + half) >> (shift - 2), &w.yh, &w.yl);
     return w;
 }
-// component value h 2^32 + l of a table of scale `shift`, as a double
+// component value h 2^32 + l of a table of scale `shift` (1 to 5), as a double.
+// The FP64 path is bound by FP64 issue, so this is integer work: a component is
+// 0 or, as sin(2 pi / 2^13) > 2^-11, at least 2^48.
 FX_HD double fx_twiddle_value(int32_t h, int32_t l, int shift)
 {
-    return ((double)h * 4294967296.0 + (double)l) / (double)(1ULL << (64 - shift));
+    const int64_t X = (int64_t)h * 4294967296LL + l;
+    int32_t big = -1;
+    const double v = fx_to_big(X, shift - 64, big);
+    return X == 0 ? 0.0 : v;
 }
 
 }  // namespace fft3d

@@ -1093,7 +1093,7 @@ template <typename R, int M, bool C2R> __host__ __device__ constexpr bool z_l2pf
 
 // Rotation factor rot[k] = exp(-2 pi i k / 2M) of slot i (k = j + i NT).
 // Float lines load rot[j] once and multiply by the slot's constant
-// exp(-i pi i / E) (NT / 2M = 1 / 2E); double lines load every factor.
+// exp(-i pi i / E) (NT / 2M = 1 / 2E).
 template <typename R, int E, int I>
 __device__ __forceinline__ typename cvec<R>::T z_rot(typename cvec<R>::T rot_j,
                                                      const typename twvec<R>::T *__restrict__ rot, int k)
@@ -1106,11 +1106,15 @@ __device__ __forceinline__ typename cvec<R>::T z_rot(typename cvec<R>::T rot_j,
             constexpr CtCosSin w = ct_cossin_pi(-(long long)I, E);
             return cmul(rot_j, cmake<C>(R(w.c), R(w.s)));
         }
-    } else if constexpr (sizeof(R) == 8) {
-        return cmake<C>(fx_twiddle_value(rot[k].xh, rot[k].xl, 2), fx_twiddle_value(rot[k].yh, rot[k].yl, 2));
     } else {
         return __ldg(rot + k);
     }
+}
+// Double lines: rot[k] / 2, as if the table's scale were one smaller.
+__device__ __forceinline__ double2 z_half_rot(const fxtw *__restrict__ rot, int k)
+{
+    const fxtw w = tw_read<false>(rot, k);
+    return make_double2(fx_twiddle_value(w.xh, w.xl, kFxRotShift - 1), fx_twiddle_value(w.yh, w.yl, kFxRotShift - 1));
 }
 
 // LPB lines starting at line0, NT = M / E threads per line.  R2C: load the
@@ -1182,8 +1186,8 @@ __device__ __forceinline__ void zr2c_lines(const ZArgs &a, int64_t line0, unsign
             const int k = j + i * NT;
             const C z = ex.get(pad_row<P, LR>(j, i * NT));
             const C zm = (i == 0 && j == 0) ? z : ex.get(pad_row<P, LREV>(M - j, -i * NT));
-            const C r = z_rot<R, E, i>(rot_j, rot, k);
-            const C A = cmake<C>(R(0.5) + R(0.5) * r.y, R(-0.5) * r.x), B = cmake<C>(R(0.5) - R(0.5) * r.y, R(0.5) * r.x);
+            const C h = z_half_rot(rot, k);
+            const C A = cmake<C>(R(0.5) + h.y, -h.x), B = cmake<C>(R(0.5) - h.y, h.x);
             // A z + B conj(zm)
             C x = cmake<C>(fma(A.x, z.x, fma(-A.y, z.y, fma(B.x, zm.x, B.y * zm.y))),
                            fma(A.x, z.y, fma(A.y, z.x, fma(B.y, zm.x, -B.x * zm.y))));
@@ -1302,9 +1306,8 @@ __device__ __forceinline__ void zc2r_lines(const ZArgs &a, int64_t line0, unsign
                     x = cmake<C>(we * x.x, R(0));
                     y = cmake<C>(we * y.x, R(0));
                 }
-                const C r = z_rot<R, E, i>(rot_j, rot, k);
-                const C A = cmake<C>(R(0.5) + R(0.5) * r.y, R(-0.5) * r.x),
-                        B = cmake<C>(R(0.5) - R(0.5) * r.y, R(0.5) * r.x);
+                const C h = z_half_rot(rot, k);
+                const C A = cmake<C>(R(0.5) + h.y, -h.x), B = cmake<C>(R(0.5) - h.y, h.x);
                 v[i] = cmake<C>(fma(A.x, x.x, fma(A.y, x.y, fma(B.x, y.x, -B.y * y.y))),
                                 fma(A.y, x.x, fma(-A.x, x.y, fma(B.x, y.y, B.y * y.x))));
             } else {
