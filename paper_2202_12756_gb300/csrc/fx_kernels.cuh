@@ -133,12 +133,13 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
         }
         __syncthreads();
         g = code[c];
-        if (!__all_sync(0xffffffffu, fx_code_ok(g))) {  // every warp holds every column of the tile
-            __syncthreads();
-            col_tile_slow<L, E, W, INV>(a, blockIdx.x, smem_raw, tw);
-            return;
+        if (!__all_sync(0xffffffffu, fx_in_range(g))) {  // every warp holds every column of the tile
+            if (__syncthreads_or(!fx_in_range(g) && fx_unfit<E>(g, r))) {
+                col_tile_slow<L, E, W, INV>(a, blockIdx.x, smem_raw, tw);
+                return;
+            }
+            g = g == 0 ? kFxZeroCode : g;
         }
-        g = g == 0 ? kFxZeroCode : g;
 #pragma unroll
         for (int i = 0; i < E; ++i)
             v[i] = fx_make(fx_from(INV ? r[i].y : r[i].x, g, kFxBits), fx_from(INV ? r[i].x : r[i].y, g, kFxBits));
@@ -149,8 +150,9 @@ colpass_fx_kernel(const __grid_constant__ ColArgs a, const fxtw *__restrict__ tw
     const int e = g - 1023 - kFxBits + fx_line_shift<L, E>();
     if (valid) {
         double2 *dj = dp + (int64_t)j * ds;
-        const int64_t dstep = (int64_t)NT * ds;
-        fx_out_all<E>(v, e, [&](int i, double2 o) { dj[i * dstep] = INV ? cswap(o) : o; });
+        // below 2^29 (128 rows of a 2048 x 2048 x 2048 grid): 32 bits spare the 8-element kernels a spilled register
+        const uint32_t dstep = NT * (uint32_t)ds;
+        fx_out_all<E>(v, e, [&](int i, double2 o) { dj[(uint32_t)i * (uint64_t)dstep] = INV ? cswap(o) : o; });
     }
 }
 
@@ -171,11 +173,18 @@ template <int NT, int LPB, class Ex> __device__ __forceinline__ int fx_line_max(
     }
     return g;
 }
-// The threads that synchronise together agree.
-template <int NT> __device__ __forceinline__ bool fx_all_ok(int g)
+// Whether the line of code g, of which the thread holds v, is transformed in fixed
+// point; the threads that synchronise together agree.
+template <int NT, int LPB, int N, class Ex> __device__ __forceinline__ bool fx_line_ok(int g, const double2 *v, const Ex &ex)
 {
-    if constexpr (NT > 32) return fx_code_ok(g);
-    else return __all_sync(0xffffffffu, fx_code_ok(g));
+    if constexpr (NT > 32) {
+        if (fx_in_range(g)) return true;
+        ex.sync();  // every thread has read the code
+        return fx_line_max<NT, LPB>(fx_unfit<N>(g, v), ex) == 0;
+    } else {
+        if (__all_sync(0xffffffffu, fx_in_range(g))) return true;
+        return !__any_sync(0xffffffffu, !fx_in_range(g) && fx_unfit<N>(g, v));
+    }
 }
 
 template <int M, int E, int LPB>
@@ -215,7 +224,7 @@ __device__ __forceinline__ void zr2c_fx_lines(const ZArgs &a, int64_t line0, uns
 #pragma unroll
         for (int i = 0; i < E; ++i) r[i] = active ? in[j + i * NT] : cmake<double2>(0.0, 0.0);
         g = fx_line_max<NT, LPB>(fx_thread_code<E>(r), ex);
-        if (!fx_all_ok<NT>(g)) {
+        if (!fx_line_ok<NT, LPB, E>(g, r, ex)) {
             zr2c_slow<M, E, LPB>(a, line0, smem, tw, rot);
             return;
         }
@@ -309,7 +318,7 @@ __device__ __forceinline__ void zc2r_fx_lines(const ZArgs &a, int64_t line0, uns
             r[E] = cmake<double2>(a.scale_edge * r[E].x, 0.0);
         }
         g = fx_line_max<NT, LPB>(fx_thread_code<E + 1>(r), ex);
-        if (!fx_all_ok<NT>(g)) {
+        if (!fx_line_ok<NT, LPB, E + 1>(g, r, ex)) {
             zc2r_slow<M, E, LPB>(a, line0, smem, tw, rot);
             return;
         }
@@ -401,7 +410,7 @@ __device__ __forceinline__ void zr2c_fx_pairs(const ZArgs &a, int64_t line0, uns
 #pragma unroll
         for (int i = 0; i < E; ++i) r[i] = cmake<double2>(act0 ? in0[j + i * NT] : 0.0, act1 ? in1[j + i * NT] : 0.0);
         g = fx_line_max<NT, PPB>(fx_thread_code<E>(r), ex);
-        if (!fx_all_ok<NT>(g)) {
+        if (!fx_line_ok<NT, PPB, E>(g, r, ex)) {
             zr2c_slow<M, E, LPB>(a, line0, smem, tw, nullptr);
             return;
         }
@@ -482,7 +491,7 @@ __device__ __forceinline__ void zc2r_fx_pairs(const ZArgs &a, int64_t line0, uns
         }
         // a thread's transform inputs have at most twice this L1 norm (its own entries and their mirror images)
         g = fx_line_max<NT, PPB>(fx_thread_code<E + 1>(r), ex);
-        if (!fx_all_ok<NT>(g)) {
+        if (!fx_line_ok<NT, PPB, E + 1>(g, r, ex)) {
             zc2r_slow<M, E, LPB>(a, line0, smem, tw, nullptr);
             return;
         }

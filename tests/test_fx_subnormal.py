@@ -1,6 +1,6 @@
 """Scale codes of double lines at the lower end of the exponent range
-(csrc/fx_math.cuh), on the host: only a line of zeros has the code of zeros; any
-other line whose values lie below 2^-895 has a code outside the conversions' range."""
+(csrc/fx_math.cuh), on the host: of the lines whose values lie below 2^-895 only one of
+zeros is transformed in fixed point."""
 import os
 import shutil
 import subprocess
@@ -15,25 +15,30 @@ PROGRAM = r"""
 #include <cmath>
 #include <cstdio>
 using namespace fft3d;
+template <int N> static bool fixed(const double2 *v)
+{
+    const int g = fx_thread_code<N>(v);
+    return fx_in_range(g) || !fx_unfit<N>(g, v);
+}
 template <int N> static int wrong()
 {
     int bad = 0;
     double2 v[N];
     for (double2 &z : v) z = make_double2(0.0, -0.0);
-    if (fx_thread_code<N>(v) != 0) ++bad;
+    if (fx_thread_code<N>(v) != 0 || !fixed<N>(v)) ++bad;
     for (int k = -1074; k <= -1000; ++k)
         for (int i = 0; i < 2 * N; ++i)
             for (int s = -1; s <= 1; s += 2) {
                 for (double2 &z : v) z = make_double2(0.0, -0.0);
                 (i < N ? v[i].x : v[i - N].y) = ldexp(s, k);
-                if (fx_code_ok(fx_thread_code<N>(v))) ++bad;
+                if (fixed<N>(v)) ++bad;
             }
     // beside an ordinary value a subnormal one makes no difference
     for (double2 &z : v) z = make_double2(0.0, 0.0);
     v[0].x = 1.0;
     const int g = fx_thread_code<N>(v);
     v[0].y = ldexp(1.0, -1074);
-    if (fx_thread_code<N>(v) != g || !fx_code_ok(g)) ++bad;
+    if (fx_thread_code<N>(v) != g || !fixed<N>(v)) ++bad;
     return bad;
 }
 int main()
