@@ -9,27 +9,15 @@
 
 namespace fft3d {
 
+// Block-size cap of a one-tile-per-block float column pass: 1024 threads, so
+// that a tile row stays one 128-byte segment even at 24 elements per thread, at
+// the price of a few spilled registers there.
 #ifndef FFT3D_COL_MAXT_F32
 #define FFT3D_COL_MAXT_F32 1024
-#endif
-#ifndef FFT3D_COL_MAXT_F64
-#define FFT3D_COL_MAXT_F64 256
 #endif
 #ifndef FFT3D_Z_THREADS
 #define FFT3D_Z_THREADS 256
 #endif
-
-// Block-size cap of a one-tile-per-block column pass: 1024 threads for float
-// (so a tile row stays one 128-byte segment even at 24 elements per thread,
-// at the price of a few spilled registers there), 256 for double: at 128
-// registers a thread two such blocks share an SM, so that one loads, stores or
-// waits at a barrier while the other computes.  Measured on GB300 at 1024^3
-// (4-column tiles, 64-byte row segments): column passes 6.7 ms, against 8.4-8.7
-// with one block of 512 threads and 8-column tiles.
-template <typename R, int L> __host__ __device__ constexpr int col_max_threads()
-{
-    return sizeof(R) == 4 ? FFT3D_COL_MAXT_F32 : (line_E(L) <= 16 ? FFT3D_COL_MAXT_F64 : 256);
-}
 
 // float columns of 2^k >= 1024 points use the persistent pipelined kernel
 // with 32 elements per thread (radix-32 stages: one exchange at 1024 points);
@@ -89,9 +77,12 @@ template <typename R, int L> __host__ __device__ constexpr int col_E()
 }
 
 // Columns per tile of a fixed-point column pass along axis AX: 256 threads a
-// block (128 for 3 * 2^k <= 384, whose 24-element threads then keep 168
-// registers instead of spilling: 192-point columns 0.064 -> 0.053 ms at
-// 192 x 128 x 384), at most a warp's worth.  The x-pass of 512 points takes 8
+// block, as at 128 registers a thread two such blocks share an SM and one loads,
+// stores or waits at a barrier while the other computes (1024^3: column passes
+// 6.7 ms, 8.4-8.7 with one block of 512 threads and 8-column tiles); 128 for
+// 3 * 2^k <= 384, whose 24-element threads then keep 168 registers instead of
+// spilling (192-point columns 0.064 -> 0.053 ms at 192 x 128 x 384); at most a
+// warp's worth.  The x-pass of 512 points takes 8
 // columns and 512 threads: its rows lie N1 (N2/2+1) entries apart, where a copy
 // in 64-byte row segments reaches 3.1-3.7 TB/s and one in 128-byte segments
 // 5.7-6 (512^3: 0.70 -> 0.68 ms, 512 x 512 x 2048: 3.03 -> 2.67; the y-pass
@@ -114,7 +105,7 @@ template <typename R, int L, int AX = 1> __host__ __device__ constexpr int col_W
         return w;
     }
     if (col_fixed<R, L>()) return col_fx_W<R, L, AX>();
-    while (w > 1 && (w * (L / col_E<R, L>()) > col_max_threads<R, L>() ||
+    while (w > 1 && (w * (L / col_E<R, L>()) > FFT3D_COL_MAXT_F32 ||
                      (size_t)L * w * sizeof(typename cvec<R>::T) > 200 * 1024))
         w /= 2;
     return w;
