@@ -71,11 +71,10 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "src": "fallback"}
 
 
-def fp64_op_counts(workload):
-    """FP64 instructions per complex half-spectrum element of each pass
-    (dadd, dmul, dfma; counted by ncu on a small case of the same line
-    lengths), or None when the kernels changed since they were counted."""
-    p = os.path.join(ROOT, "profiles", "fp64_ops.json")
+def captured(name, workload):
+    """Entry of a committed ncu summary, or None when the kernels changed
+    since it was captured."""
+    p = os.path.join(ROOT, "profiles", name)
     if not os.path.exists(p):
         return None
     d = json.load(open(p))
@@ -84,9 +83,27 @@ def fp64_op_counts(workload):
     return d.get("workloads", {}).get(workload)
 
 
+def issue_roofline(stats, counts, sms, sm_mhz, units):
+    """Instruction-issue roofline of the slowest FP64 pass, which runs on the
+    integer pipes: warp instructions per complex half-spectrum element (counted
+    by ncu on this workload) times the elements of a launch over its mean launch
+    time, against one instruction per clock of each SM quarter."""
+    if not stats:
+        return None
+    top = max(stats, key=lambda s: s["total_ms"])
+    avg_ms = top["total_ms"] / top["launches"]
+    peak = None if not sm_mhz else sms * 4 * sm_mhz * 1e-3
+    c = (counts or {}).get(top["name"])
+    achieved = None if c is None else c * units / (avg_ms * 1e-3) / 1e9
+    return {"bound": "instruction issue", "kernel": top["name"], "avg_launch_ms": round(avg_ms, 4),
+            "peak": None if peak is None else round(peak, 1), "unit": "G warp instructions/s",
+            "warp_inst_per_element": c, "achieved": None if achieved is None else round(achieved, 1),
+            "frac": None if achieved is None or peak is None else round(achieved / peak, 4)}
+
+
 def fp64_roofline(stats, ops, peak, units):
-    """FP64-ALU roofline of the slowest FP64 pass: its FP64 instructions per
-    launch (ops per element x units) over its mean launch time, against the
+    """FP64-ALU roofline of the slowest pass that runs in FP64 arithmetic: its
+    FP64 instructions per launch (ops per element x units) over its mean launch time, against the
     measured FP64 instruction rate (the best of FMA, add and multiply; each
     takes one FP64 issue slot)."""
     if not stats or not peak:
@@ -111,15 +128,8 @@ def fp64_roofline(stats, ops, peak, units):
 
 
 def ncu_traffic(workload):
-    """Per-launch DRAM bytes of each pass from the committed ncu summary, or
-    None when the kernels changed since it was captured."""
-    p = os.path.join(ROOT, "profiles", "ncu_traffic.json")
-    if not os.path.exists(p):
-        return None
-    d = json.load(open(p))
-    if d.get("kernel_hash") != kernel_sources_hash():
-        return None
-    return d.get("workloads", {}).get(workload)
+    """Per-launch DRAM bytes of each pass from the committed ncu summary."""
+    return captured("ncu_traffic.json", workload)
 
 
 class ClockSampler:
@@ -531,7 +541,7 @@ def run_ours(args):
     # ---- reference point: cuFFT through torch.fft on the same field (rank 0)
     torch_ref = torch_fft_reference(buf32, grid, dev) if rank == 0 else None
 
-    # ---- FP64 pair (same field), then its per-pass times and the FP64 roof
+    # ---- FP64 pair (same field), then its per-pass times and the FP64 rate of this GPU
     steps64 = max(2, args.steps // 10)
     ms64, launches64, _, _ = time_pairs(plan64, buf64, steps64, args.warmup, dev, pg)
     ms64 = max_over_ranks(ms64, pg, dev)
@@ -633,7 +643,10 @@ def run_ours(args):
                  "gflops": round(flops * world / (t64 * 1e-3) / 1e9, 1),
                  "hbm_gbs": round(2 * pass_bytes(n0, n1, n, 8) / (t64 * 1e-3) / 1e9, 1),
                  "per_pass_ms": per_pass(stats64, 3),
-                 "roofline": fp64_roofline(stats64, fp64_op_counts(f"{n0}x{n1}x{n} f64"), fp64_peak, units),
+                 "roofline": issue_roofline(stats64, captured("fx_issue.json", f"{n0}x{n1}x{n} f64"),
+                                            torch.cuda.get_device_properties(dev).multi_processor_count,
+                                            (clk or {}).get("sm_mhz"), units),
+                 "fp64_rate_gflops": {k: round(v, 1) for k, v in fp64_peak.items()},
                  "fp32_speedup": round(t64 / t_step, 2)},
         "e2e": {"value": round(e2e_val, 1), "unit": UNIT, "ms_per_step": round(ms_e2e, 3),
                 "h2d_bytes_per_step": io_bytes, "d2h_bytes_per_step": io_bytes,

@@ -56,7 +56,10 @@ typedef struct fft3d_plan_s *fft3d_plan;
 
 enum fft3d_dtype {
     FFT3D_F32 = 0, /* float storage and arithmetic, twiddles generated in FP64 */
-    FFT3D_F64 = 1  /* double storage and arithmetic */
+    /* double storage; lines of 8 points and more are transformed in 64-bit block fixed
+     * point (errors as in double arithmetic or smaller), or in double arithmetic where
+     * they hold non-finite values or lie near the ends of the exponent range */
+    FFT3D_F64 = 1
 };
 
 enum fft3d_status {
@@ -280,10 +283,11 @@ int fft3d_exec_c2r_noalloc(const void *in_cplx, void *out_real, int64_t n0, int6
 int fft3d_noalloc_status(int *device_error);
 
 /*
- * FP64 throughput of the current device, measured: the roof of the FP64
- * passes, which on GB300 are bound by FP64 add / multiply issue rather than
- * by HBM (the paper compares single and double precision in Sec. 4, Table
- * 3).  Runs three short kernels (FMA, add and multiply chains that fill every
+ * FP64 throughput of the current device, measured: the roof of double lines
+ * that are transformed in FP64 arithmetic (see FFT3D_F64), which on GB300 are
+ * bound by FP64 add / multiply issue rather than by HBM; the others run on the
+ * integer pipes for that reason (the paper compares single and double precision
+ * in Sec. 4, Table 3).  Runs three short kernels (FMA, add and multiply chains that fill every
  * SM) on a private stream and synchronises; stores the best of three timed
  * launches of each in GFLOP/s (an FMA counts two flops, an add or multiply
  * one).  A diagnostic for the bench; it touches no plan or user memory.

@@ -1,7 +1,7 @@
 // FP64 arithmetic throughput of the current GPU, measured in place: the roof
-// that bounds the FP64 passes (the paper's double-precision runs, Sec. 4,
-// Table 3), which on GB300 are limited by FP64 add / multiply issue rather
-// than by HBM.
+// of the double lines that are transformed in FP64 arithmetic, which on GB300
+// are limited by FP64 add / multiply issue rather than by HBM (the others run
+// on the integer pipes; the paper's double-precision runs: Sec. 4, Table 3).
 //
 // Each thread runs 8 independent dependency chains of one FP64 operation
 // (FMA, add or multiply), so the FP64 units, not latency, set the rate; the

@@ -33,8 +33,8 @@ namespace fft3d {
 
 // Start of every pass kernel: a pass is launched while the kernel before it on
 // the stream ends (launch_pass; earlier where that one releases it) and waits
-// here until that kernel has completed and its writes are visible.  All blocks wait, so completion
-// carries over from kernel to kernel.
+// here until that kernel has completed and its writes are visible.  All blocks
+// wait, so completion carries over from kernel to kernel.
 __device__ __forceinline__ void pass_begin() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 // ------------------------------------------------------------ layouts
