@@ -5,7 +5,7 @@
 // double range) runs the FP64 pass instead, from the same twiddle tables.
 //
 // Measured on GB300 in place (FP64 arithmetic -> fixed point): 1024^3 pair
-// 190.1 -> 31.8 ms, 512^3 21.6 -> 3.54 ms; relative L2 error of one transform
+// 190.3 -> 31.7 ms, 512^3 21.6 -> 3.58 ms; relative L2 error of one transform
 // against extended precision, over line lengths, noise and single-spike lines:
 // 1.6-2.8e-16 -> 0.5-1.8e-16.  The FP64 pass in place of it keeps the speed of
 // kernels of FP64 arithmetic alone: 512^3 pair with one infinity 22.0 ms (21.6).
